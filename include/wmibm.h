@@ -259,23 +259,24 @@ int wmibm_mask(wmibm_handle *h, void *u, void *v, void *w, const void *const gra
 /*
  * wmibm_step - wmibm_wall_stress, wmibm_force and wmibm_mask in that order on
  * one stream: one pass of the whole per-step stress stage, with the same results
- * as the three calls.  Where the pipelined stencil takes the grid (see
- * wmibm_force_mask) and tuning.force_path is not 3, it is ONE cooperative launch:
- * in every block the consumer warps first evaluate the block's share of the
- * band nodes and solid runs while the producer streams the stencil stages that
- * read no band or solid node; stages that do wait (bounded) until every block
- * has finished its wall share; the body mask follows the forcing.  Otherwise
- * it is two launches (the wall-model kernel, then the force + mask kernel as
- * its programmatic dependent).  A cooperative launch needs all its blocks
- * resident: it fails with ECUDA if another context holds the SMs it needs.
+ * as the three calls.  By default (tuning.force_path 0 or 3) it is two launches
+ * where the pipelined stencil takes the grid (see wmibm_force_mask): the
+ * wall-model kernel, then the force + mask kernel as its programmatic dependent,
+ * which streams the stages that read no band or solid node meanwhile.  With
+ * force_path 1, 4, 5 or 6 it is ONE cooperative launch there: in every block the
+ * consumer warps (1) first evaluate the block's share of the band nodes and solid
+ * runs while the producer streams the clean stages; stages that read them wait
+ * (bounded) until every block has finished its wall share; the body mask follows
+ * the forcing.  A cooperative launch needs all its blocks resident: it fails with
+ * ECUDA if another context holds the SMs it needs.
  */
 int wmibm_step(wmibm_handle *h, void *u, void *v, void *w, void *const tau[6], void *fx, void *fy, void *fz,
                const void *const gradp[3], double dt, wmibm_band_stats *stats, void *stream);
 
 /*
  * wmibm_wall_stress_force - wmibm_wall_stress followed by wmibm_force on one
- * stream (same arguments and results as the two calls); one cooperative launch
- * under the same conditions as wmibm_step (without the body mask).
+ * stream (same arguments and results as the two calls), in the launches that
+ * wmibm_step takes (without the body mask).
  */
 int wmibm_wall_stress_force(wmibm_handle *h, const void *u, const void *v, const void *w, void *const tau[6],
                             void *fx, void *fy, void *fz, wmibm_band_stats *stats, void *stream);
@@ -296,7 +297,7 @@ int wmibm_force_mask(wmibm_handle *h, const void *const tau[6], void *fx, void *
  * mean "choose automatically".
  */
 typedef struct wmibm_tuning {
-    int32_t force_path;       /* 0 auto, 1 bulk-copy pipeline only, 2 direct-load kernel only,
+    int32_t force_path;       /* 0 auto (as 3), 1 bulk-copy pipeline only, 2 direct-load kernel only,
                                  3 bulk-copy pipeline with the wall model always in a kernel of its
                                  own (no single-launch step), 4 as 1 with the single-launch step's
                                  wall model in dedicated blocks (one per SM) instead of a share of

@@ -65,10 +65,8 @@ void force_default_tile(const wmibm_handle *h, int *bx, int *by, int *kc);
 int force_any(wmibm_handle *h, const void *const tau[6], void *fx, void *fy, void *fz, cudaStream_t stream);
 bool stencil_config(const wmibm_handle *h, const void *const tau[6], void *const f[3], StencilConfig *out);
 int stencil_force_mask(wmibm_handle *h, void *u, void *v, void *w, const void *const tau[6], void *const f[3],
-                       const void *const gradp[3], double dt, const StencilConfig &c, bool pdl, cudaStream_t stream,
-                       wmibm_band_stats *emit);
-int stencil_force(wmibm_handle *h, const void *const tau[6], void *const f[3], const StencilConfig &c,
-                  cudaStream_t stream, wmibm_band_stats *emit);
+                       const void *const gradp[3], double dt, int do_mask, const StencilConfig &c, bool pdl,
+                       cudaStream_t stream, wmibm_band_stats *emit);
 int wall_model(wmibm_handle *h, const void *u, const void *v, const void *w, void *const tau[6],
                wmibm_band_stats *stats, const void *logz0, cudaStream_t stream, bool emit);
 int mask_impl(wmibm_handle *h, void *u, void *v, void *w, const void *const gradp[3], double dt, cudaStream_t stream);
@@ -89,10 +87,8 @@ static int two_launch_step(wmibm_handle *h, const void *u, const void *v, const 
     if (stencil_config(h, (const void *const *)tau, f, &c)) {
         int st = wall_model(h, u, v, w, tau, stats, h->logz0, stream, false);
         if (st) return st;
-        if (do_mask)
-            return stencil_force_mask(h, const_cast<void *>(u), const_cast<void *>(v), const_cast<void *>(w),
-                                      (const void *const *)tau, f, gradp, dt, c, true, stream, stats);
-        return stencil_force(h, (const void *const *)tau, f, c, stream, stats);
+        return stencil_force_mask(h, const_cast<void *>(u), const_cast<void *>(v), const_cast<void *>(w),
+                                  (const void *const *)tau, f, gradp, dt, do_mask, c, true, stream, stats);
     }
     int st = wall_model(h, u, v, w, tau, stats, h->logz0, stream, true);
     if (st) return st;
@@ -101,14 +97,19 @@ static int two_launch_step(wmibm_handle *h, const void *u, const void *v, const 
     return mask_impl(h, const_cast<void *>(u), const_cast<void *>(v), const_cast<void *>(w), gradp, dt, stream);
 }
 
-// Wall stress + force (+ mask): one cooperative launch where the pipelined
-// stencil takes the grid and the tuning allows it; else returns 1 and does nothing.
+// Wall stress + force (+ mask) in one cooperative launch, where the tuning asks for
+// one and the pipelined stencil takes the grid; else *done stays 0 and nothing is
+// done.  Untuned handles take two launches: the stencil streams its clean units
+// beside the wall kernel's tail, and neither holds the other's registers (step in
+// us, one launch against two: 64^3 17.7 / 14.6, 192 x 96 x 96 26.9 / 23.1, cubes
+// 256 x 128 x 128 49.6 / 41.6, hill 512 x 256 x 256 237 / 228; FP64: 32^3 28.8 /
+// 28.3, 256 x 128 x 128 219 / 205).
 static int try_fused(wmibm_handle *h, void *u, void *v, void *w, void *const tau[6], void *fx, void *fy, void *fz,
                      const void *const gradp[3], double dt, int do_mask, wmibm_band_stats *stats,
                      cudaStream_t stream, int *done)
 {
     *done = 0;
-    if (h->tuning.force_path == 3) return WMIBM_OK;
+    if (h->tuning.force_path == 0 || h->tuning.force_path == 3) return WMIBM_OK;
     void *const f[3] = {fx, fy, fz};
     StencilConfig c;
     if (!stencil_config(h, (const void *const *)tau, f, &c)) return WMIBM_OK;
@@ -125,7 +126,7 @@ int force_mask_impl(wmibm_handle *h, void *u, void *v, void *w, void *const tau[
     StencilConfig c;
     if (stencil_config(h, (const void *const *)tau, f, &c)) {
         if (do_mask)
-            return stencil_force_mask(h, u, v, w, (const void *const *)tau, f, gradp, dt, c, pdl, stream, nullptr);
+            return stencil_force_mask(h, u, v, w, (const void *const *)tau, f, gradp, dt, 1, c, pdl, stream, nullptr);
         return force_any(h, (const void *const *)tau, fx, fy, fz, stream);
     }
     int st = force_any(h, (const void *const *)tau, fx, fy, fz, stream);

@@ -552,6 +552,8 @@ __device__ void produce(const KParams<T> &p, T *ring_a, T *ring_b, uint64_t *ful
             }
         }
     }
+    // a launch without dirty units ends after the wall kernel all the same: what follows it in the stream relies on both
+    if (MODE == kAfterWall && !released) wait_wall_kernel();
     if (!it.done) {
         // gave up: let the copies already issued land before the block exits
         const uint32_t first = g > SA ? g - SA : 0;
@@ -1938,8 +1940,14 @@ bool stencil_config(const wmibm_handle *h, const void *const tau[6], void *const
     if (c.rows == 0) {
         // default: the shape the autotuner keeps for the measured grids (nx 256 and
         // 512): 4-row strips and two stages; narrower strips where the rows do not
-        // divide ny or the rings would not fit
+        // divide ny or the rings would not fit.  FP64, bound by its arithmetic, takes
+        // two rows where they leave room for two blocks per SM and four do not (256 x 128 x 128: 194
+        // against 204 us; FP32 at nx = 512 stays with four, 228 against 251)
         c.rows = 4;
+        const int default_stages = c.stages > 0 ? c.stages : 2;
+        if (es == 8 && ring_bytes(4, default_stages) + 256 > 113 * 1024 &&
+            ring_bytes(2, default_stages) + 256 <= 113 * 1024)
+            c.rows = 2;
         while (c.rows > 1 && (h->ny % c.rows != 0 || h->ny < c.rows + 2 ||
                               ring_bytes(c.rows, c.stages > 0 ? c.stages : 2) + 256 > (size_t)kMaxDynSmem))
             c.rows /= 2;
@@ -1987,11 +1995,12 @@ int stencil_force(wmibm_handle *h, const void *const tau[6], void *const f[3], c
     return launch_stencil<float, float, kPlain>(h, p, c, stream, false, h->nx);
 }
 
-// The pipelined stencil followed, in the same launch, by the body mask (Eq. 27).
-// With pdl the launch is a programmatic dependent of the preceding kernel.
+// The pipelined stencil after a wall launch, followed with do_mask, in the same
+// launch, by the body mask (Eq. 27).  With pdl the launch is a programmatic
+// dependent of the preceding kernel.
 int stencil_force_mask(wmibm_handle *h, void *u, void *v, void *w, const void *const tau[6], void *const f[3],
-                       const void *const gradp[3], double dt, const StencilConfig &c, bool pdl, cudaStream_t stream,
-                       wmibm_band_stats *emit)
+                       const void *const gradp[3], double dt, int do_mask, const StencilConfig &c, bool pdl,
+                       cudaStream_t stream, wmibm_band_stats *emit)
 {
     if (h->dtype == WMIBM_F64) {
         KParams<double> p;
@@ -1999,7 +2008,7 @@ int stencil_force_mask(wmibm_handle *h, void *u, void *v, void *w, const void *c
         single_params<double>(h, p, true);
         p.stages = c.stages;
         p.ncons = c.consumer_warps;
-        p.do_mask = 1;
+        p.do_mask = do_mask;
         p.stats = emit;
         p.emit_stats = emit != nullptr;
         return launch_stencil<double, double, kAfterWall>(h, p, c, stream, pdl, h->nx);
@@ -2009,7 +2018,7 @@ int stencil_force_mask(wmibm_handle *h, void *u, void *v, void *w, const void *c
     single_params<float>(h, p, true);
     p.stages = c.stages;
     p.ncons = c.consumer_warps;
-    p.do_mask = 1;
+    p.do_mask = do_mask;
     p.stats = emit;
     p.emit_stats = emit != nullptr;
     if (h->vel_dtype == WMIBM_BF16)
