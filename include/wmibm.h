@@ -282,6 +282,27 @@ int wmibm_wall_stress_force(wmibm_handle *h, const void *u, const void *v, const
                             void *fx, void *fy, void *fz, wmibm_band_stats *stats, void *stream);
 
 /*
+ * wmibm_wall_stress_force_from - the forcing of wmibm_wall_stress_force from
+ * stresses that are left as they are (what differentiating the stage needs): the
+ * entries that the wall model writes go to a work buffer, of which only the levels
+ * with band or solid nodes (and their neighbours) are filled.
+ *   tau      : DEVICE, 6 stress fields (dtype), read only
+ *   work     : DEVICE, 16-byte aligned, at least wmibm_stage_work_bytes(h, tau, fx,
+ *              fy, fz) bytes (NULL where that is 0); overlaps no other argument.
+ *              Its contents afterwards mean nothing to a caller
+ *   others   : as in wmibm_wall_stress_force
+ * Two launches and the copy, whatever force_path is set to.
+ * Errors: EINVAL, ESTATE, ECUDA.
+ */
+int wmibm_wall_stress_force_from(wmibm_handle *h, const void *u, const void *v, const void *w,
+                                 const void *const tau[6], void *work, int64_t work_bytes, void *fx, void *fy, void *fz,
+                                 wmibm_band_stats *stats, void *stream);
+
+/* Bytes of that call's work buffer for these fields (their alignment counts) and the handle's tuning; -1 for a bad argument. */
+int64_t wmibm_stage_work_bytes(const wmibm_handle *h, const void *const tau[6], const void *fx, const void *fy,
+                               const void *fz);
+
+/*
  * wmibm_force_mask - wmibm_force followed by wmibm_mask, in one launch where the
  * grid allows the pipelined stencil (nx a multiple of 4 for F32 or 2 for F64,
  * ny >= 3, 16-byte aligned stress and force buffers, full x-rows that fit the

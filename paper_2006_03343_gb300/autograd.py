@@ -15,9 +15,10 @@ class WallStressForce(torch.autograd.Function):
     @staticmethod
     def forward(ctx, handle, u, v, w, logz0, txx, txy, tyy, tzz, txz, tyz):
         handle.set_log_z0(logz0)
-        tau = [t.detach().clone() for t in (txx, txy, tyy, tzz, txz, tyz)]
+        # the stresses are read in place; views that are not contiguous go through a copy
+        tau = [t if t.is_contiguous() else t.detach().clone() for t in (txx, txy, tyy, tzz, txz, tyz)]
         f = [torch.empty(handle.shape, dtype=handle.torch_dtype, device=handle.device) for _ in range(3)]
-        handle.wall_stress_force(u.detach(), v.detach(), w.detach(), tau, f)
+        handle.wall_stress_force_from(u, v, w, tau, f)
         ctx.handle = handle
         ctx.save_for_backward(u, v, w, logz0)
         return f[0], f[1], f[2]
@@ -30,7 +31,7 @@ class WallStressForce(torch.autograd.Function):
              for t in (gx, gy, gz)]
         h.set_log_z0(logz0)
         du, dv, dw, ds = (torch.empty(h.shape, dtype=h.torch_dtype, device=h.device) for _ in range(4))
-        h.backward(g, (u.detach(), v.detach(), w.detach()), du, dv, dw, ds)
+        h.backward(g, (u, v, w), du, dv, dw, ds)
         cast = lambda d, x: d if d.dtype == x.dtype else d.to(x.dtype)
         return (None, cast(du, u), cast(dv, v), cast(dw, w), ds) + (None,) * 6
 

@@ -10,6 +10,8 @@ namespace wmibm {
 template <typename T>
 struct Member {
     const T *tau[6];              // txx txy tyy tzz txz tyz (the wall kernel writes band / solid entries)
+    const T *tin[6];              // the stresses that clean units read: tau, or the caller's fields where tau
+                                  // holds only the levels that dirty units read
     T *f[3];
     void *u, *v, *w;
     int32_t nx, ny, nz, nstrips, rows;   // rows: x-rows per strip of the stencil

@@ -82,7 +82,7 @@ __device__ __forceinline__ void stg(double *p, const Pack<double> &x)
 // constant-offset loads, so that nothing is copied to local memory).
 template <typename T>
 struct ProdView {
-    const T *tau[6];
+    const T *tau[6], *tin[6];
     int32_t nx, ny, nz, ty;
 };
 
@@ -102,11 +102,15 @@ __device__ __forceinline__ void load_prod(const KParams<T> &p, int m, ProdView<T
     if (p.nmembers == 1) {
         v.tau[0] = p.one.tau[0]; v.tau[1] = p.one.tau[1]; v.tau[2] = p.one.tau[2];
         v.tau[3] = p.one.tau[3]; v.tau[4] = p.one.tau[4]; v.tau[5] = p.one.tau[5];
+        v.tin[0] = p.one.tin[0]; v.tin[1] = p.one.tin[1]; v.tin[2] = p.one.tin[2];
+        v.tin[3] = p.one.tin[3]; v.tin[4] = p.one.tin[4]; v.tin[5] = p.one.tin[5];
         v.nx = p.one.nx; v.ny = p.one.ny; v.nz = p.one.nz; v.ty = p.one.rows;
     } else {
         const Member<T> *mm = p.list + m;
         v.tau[0] = mm->tau[0]; v.tau[1] = mm->tau[1]; v.tau[2] = mm->tau[2];
         v.tau[3] = mm->tau[3]; v.tau[4] = mm->tau[4]; v.tau[5] = mm->tau[5];
+        v.tin[0] = mm->tau[0]; v.tin[1] = mm->tau[1]; v.tin[2] = mm->tau[2];
+        v.tin[3] = mm->tau[3]; v.tin[4] = mm->tau[4]; v.tin[5] = mm->tau[5];
         v.nx = mm->nx; v.ny = mm->ny; v.nz = mm->nz; v.ty = mm->rows;
     }
 }
@@ -530,8 +534,10 @@ __device__ void produce(const KParams<T> &p, T *ring_a, T *ring_b, uint64_t *ful
                 bulk_g2s(dst, base + (int64_t)jstart * nx, (uint32_t)cnt * row_bytes, &full[b]);
             }
         };
-        const T *const txx = v.tau[0], *const txy = v.tau[1], *const tyy = v.tau[2];
-        const T *const tzz = v.tau[3], *const txz = v.tau[4], *const tyz = v.tau[5];
+        const bool own = it.dirty;
+        const T *const txx = own ? v.tau[0] : v.tin[0], *const txy = own ? v.tau[1] : v.tin[1];
+        const T *const tyy = own ? v.tau[2] : v.tin[2], *const tzz = own ? v.tau[3] : v.tin[3];
+        const T *const txz = own ? v.tau[4] : v.tin[4], *const tyz = own ? v.tau[5] : v.tin[5];
         if (it.prologue) {
             const uint32_t rows = (k > 0 ? ty : 0) + ty + (ty + 2);
             mbar_arrive_expect_tx(&full[b], rows * row_bytes);
@@ -1876,7 +1882,7 @@ template <typename T>
 void fill_member(const wmibm_handle *h, Member<T> &m, const void *const tau[6], void *const f[3], void *u, void *v,
                  void *w, const void *logz0, const void *const gradp[3], double dt, int rows)
 {
-    for (int a = 0; a < 6; ++a) m.tau[a] = (const T *)tau[a];
+    for (int a = 0; a < 6; ++a) m.tau[a] = m.tin[a] = (const T *)tau[a];
     for (int a = 0; a < 3; ++a) m.f[a] = f ? (T *)f[a] : nullptr;
     m.u = u; m.v = v; m.w = w;
     m.nx = h->nx; m.ny = h->ny; m.nz = h->nz;
@@ -2024,6 +2030,33 @@ int stencil_force_mask(wmibm_handle *h, void *u, void *v, void *w, const void *c
     if (h->vel_dtype == WMIBM_BF16)
         return launch_stencil<float, __nv_bfloat16, kAfterWall>(h, p, c, stream, pdl, h->nx);
     return launch_stencil<float, float, kAfterWall>(h, p, c, stream, pdl, h->nx);
+}
+
+// The pipelined stencil after a wall launch on `work`, which holds the levels that
+// dirty units read; clean units read the caller's stresses.
+int stencil_force_from(wmibm_handle *h, const void *const tau[6], const void *const work[6], void *const f[3],
+                       const StencilConfig &c, cudaStream_t stream, wmibm_band_stats *emit)
+{
+    if (h->dtype == WMIBM_F64) {
+        KParams<double> p;
+        fill_member<double>(h, p.one, work, f, nullptr, nullptr, nullptr, nullptr, nullptr, 0.0, c.rows);
+        for (int a = 0; a < 6; ++a) p.one.tin[a] = (const double *)tau[a];
+        single_params<double>(h, p, true);
+        p.stages = c.stages;
+        p.ncons = c.consumer_warps;
+        p.stats = emit;
+        p.emit_stats = emit != nullptr;
+        return launch_stencil<double, double, kAfterWall>(h, p, c, stream, true, h->nx);
+    }
+    KParams<float> p;
+    fill_member<float>(h, p.one, work, f, nullptr, nullptr, nullptr, nullptr, nullptr, 0.0, c.rows);
+    for (int a = 0; a < 6; ++a) p.one.tin[a] = (const float *)tau[a];
+    single_params<float>(h, p, true);
+    p.stages = c.stages;
+    p.ncons = c.consumer_warps;
+    p.stats = emit;
+    p.emit_stats = emit != nullptr;
+    return launch_stencil<float, float, kAfterWall>(h, p, c, stream, true, h->nx);
 }
 
 template <typename T, typename VEL>

@@ -30,7 +30,8 @@ EXPORTED = ("wmibm_init", "wmibm_wall_stress", "wmibm_force", "wmibm_mask", "wmi
             "wmibm_batch_set_fields", "wmibm_batch_set_tuning", "wmibm_batch_step", "wmibm_batch_traffic_bytes",
             "wmibm_batch_points", "wmibm_batch_last_error", "wmibm_batch_destroy", "wmibm_set_log_z0",
             "wmibm_backward", "wmibm_batch_wall_stress_force", "wmibm_force_spectral", "wmibm_spectral_shape", "wmibm_sgs_wall_terms", "wmibm_sgs_stress", "wmibm_sgs_force",
-            "wmibm_heightfield_sdf", "wmibm_batch_device_status")
+            "wmibm_heightfield_sdf", "wmibm_batch_device_status", "wmibm_wall_stress_force_from",
+            "wmibm_stage_work_bytes")
 
 
 class WmibmError(RuntimeError):
@@ -117,6 +118,10 @@ def load(path: Optional[str] = None):
     L.wmibm_wall_stress_force.restype = ctypes.c_int
     L.wmibm_wall_stress_noalloc.argtypes = [_VP, _VP, _VP, _VP, _PVP, _VP, _VP]
     L.wmibm_wall_stress_noalloc.restype = ctypes.c_int
+    L.wmibm_wall_stress_force_from.argtypes = [_VP, _VP, _VP, _VP, _PVP, _VP, ctypes.c_int64, _VP, _VP, _VP, _VP, _VP]
+    L.wmibm_wall_stress_force_from.restype = ctypes.c_int
+    L.wmibm_stage_work_bytes.argtypes = [_VP, _PVP, _VP, _VP, _VP]
+    L.wmibm_stage_work_bytes.restype = ctypes.c_int64
     L.wmibm_force_mask.argtypes = [_VP, _PVP, _VP, _VP, _VP, _VP, _VP, _VP, _PVP, ctypes.c_double, _VP]
     L.wmibm_force_mask.restype = ctypes.c_int
     L.wmibm_set_tuning.argtypes = [_VP, ctypes.POINTER(Tuning)]
@@ -166,10 +171,7 @@ def load(path: Optional[str] = None):
 
 
 def _ptrs(seq) -> ctypes.Array:
-    arr = (ctypes.c_void_p * len(seq))()
-    for i, t in enumerate(seq):
-        arr[i] = None if t is None else ctypes.c_void_p(_dptr(t))
-    return arr
+    return (ctypes.c_void_p * len(seq))(*[None if t is None else _dptr(t) for t in seq])
 
 
 def _dptr(t) -> int:
@@ -264,7 +266,7 @@ class Handle:
 
     def _field(self, t, vel=False):
         want = self.torch_vel_dtype if vel else self.torch_dtype
-        if t.dtype != want or not t.is_contiguous() or tuple(t.shape) != self.shape or t.device != self.device:
+        if t.dtype != want or not t.is_contiguous() or t.shape != self.shape or t.device != self.device:
             raise ValueError(f"field must be a contiguous {want} tensor of shape {self.shape} on {self.device}, "
                              f"got {t.dtype} {tuple(t.shape)} on {t.device}")
         return t
@@ -388,6 +390,23 @@ class Handle:
         self._check(self._L.wmibm_wall_stress_force(self._h, _dptr(u), _dptr(v), _dptr(w), _ptrs(tau),
                                                     _dptr(f[0]), _dptr(f[1]), _dptr(f[2]),
                                                     None if stats is None else _dptr(stats), _stream_ptr(stream)))
+
+    def wall_stress_force_from(self, u, v, w, tau, f, stats=None, stream=None):
+        """wall_stress_force from stresses that are left as they are (the entries that
+        the wall model writes go to a buffer of the call)."""
+        import torch
+        for t in (u, v, w):
+            self._field(t, vel=True)
+        for t in (*tau, *f):
+            self._field(t)
+        ptrs, fp = _ptrs(tau), [_dptr(t) for t in f]
+        work = torch.empty(int(self._L.wmibm_stage_work_bytes(self._h, ptrs, *fp)), dtype=torch.uint8,
+                           device=self.device)
+        if stream is not None:
+            work.record_stream(stream)
+        self._check(self._L.wmibm_wall_stress_force_from(self._h, _dptr(u), _dptr(v), _dptr(w), ptrs, _dptr(work),
+                                                         work.numel(), *fp, None if stats is None else _dptr(stats),
+                                                         _stream_ptr(stream)))
 
     def force_mask(self, tau, f, u, v, w, gradp=None, dt=0.0, stream=None):
         for t in list(tau) + list(f):
