@@ -175,16 +175,21 @@ def _ptrs(seq) -> ctypes.Array:
 
 
 def _dptr(t) -> int:
-    if isinstance(t, int):
-        return t
-    return int(t.data_ptr())
+    return t if isinstance(t, int) else t.data_ptr()
+
+
+_current = None         # torch's (current device, raw current stream of a device)
 
 
 def _stream_ptr(stream) -> Optional[int]:
-    import torch
-    if stream is None:
-        stream = torch.cuda.current_stream()
-    return int(stream.cuda_stream) or None
+    if stream is not None:
+        return int(stream.cuda_stream) or None
+    global _current
+    if _current is None:
+        import torch
+        # the stream's handle alone: a torch.cuda.Stream object for it takes some 4 us a call
+        _current = torch.cuda.current_device, torch._C._cuda_getCurrentRawStream
+    return _current[1](_current[0]()) or None
 
 
 def heightfield_sdf(grid, height, reach, phi_uv=None, phi_w=None, stream=None):
