@@ -925,9 +925,12 @@ __global__ void __launch_bounds__(256) k_wall(KParams<T> p)
     }
     zero_runs(mm, gw, nwarps, threadIdx.x & 31, &run0);
     if (p.sacc) {
-        // statistics into the accumulator
-        stats_block_reduce(acc, red);
-        if (threadIdx.x == 0) stats_red(acc, p.sacc);
+        // statistics into the accumulator, from the blocks that had records (in FP64
+        // a block's reduction alone takes some 5,000 cycles of its SM)
+        if ((int64_t)blockIdx.x * blockDim.x < nrec) {
+            stats_block_reduce(acc, red);
+            if (threadIdx.x == 0) stats_red(acc, p.sacc);
+        }
         if (p.emit_stats && threadIdx.x == 0) {
             __threadfence();
             s_last = atomicAdd(p.ticket, 1u) == gridDim.x - 1;
@@ -1850,7 +1853,11 @@ int launch_wall_single(wmibm_handle *h, void *const tau[6], const void *u, const
     } else if (!stats) {
         p.sacc = nullptr;
     }
-    const int wthreads = blocks ? 256 : 32 * (h->tuning.wall_warps > 0 ? h->tuning.wall_warps : 8);
+    // threads per block: a small band is spread over all SMs in blocks of few warps, so
+    // that no SM evaluates several warps' records while others have none
+    const int64_t per_sm = (h->nrec + h->sm_count - 1) / h->sm_count;
+    const int spread = (int)std::min<int64_t>(std::max<int64_t>((per_sm + 31) / 32 * 32, 32), 256);
+    const int wthreads = blocks ? 256 : (h->tuning.wall_warps > 0 ? 32 * h->tuning.wall_warps : spread);
     if (blocks == 0) {
         int wper = 0;
         const int64_t wkey = 0x100000 | wthreads | (sizeof(T) == 8 ? 0x200000 : 0);
@@ -1866,6 +1873,11 @@ int launch_wall_single(wmibm_handle *h, void *const tau[6], const void *u, const
         }
         if (h->tuning.wall_grid > 0 && h->tuning.wall_grid < wper) wper = h->tuning.wall_grid;
         blocks = (unsigned)std::min<int64_t>((int64_t)wper * h->sm_count, h->partial_blocks);
+        // no more blocks than records (one a thread) and solid runs (two a warp) ask for:
+        // idle ones hold the SMs' room and the launch's end
+        const int64_t runs = h->nruns[0] + h->nruns[1], warps = wthreads / 32;
+        const int64_t need = std::max<int64_t>((h->nrec + wthreads - 1) / wthreads, (runs + 2 * warps - 1) / (2 * warps));
+        blocks = (unsigned)std::min<int64_t>(blocks, std::max<int64_t>(need, 1));
     }
     // with the accumulator and emit, the wall kernel's last block converts the statistics
     p.emit_stats = (p.sacc && emit) ? 1 : 0;
