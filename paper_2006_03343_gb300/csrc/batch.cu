@@ -34,6 +34,7 @@ struct wmibm_batch {
     int64_t traffic[2];
     uint64_t wait_ns;
     int hold_release;
+    DirectBatch offsets;
     std::vector<unsigned char> member0;   // host copy of member 0's descriptor (a batch of one
                                           // is launched with it as the single-terrain member)
     char err[512];
@@ -118,11 +119,14 @@ bool batch_config(wmibm_batch *b, StencilConfig *out, std::vector<int> *rows_out
     return true;
 }
 
+// Levels per chunk of the direct-load stencil's blocks.
+constexpr int kDirectBatchLevels = 2;
+
 template <typename T>
 int upload_members(wmibm_batch *b, const wmibm_member_fields *fields, cudaStream_t stream)
 {
     std::vector<Member<T>> host(b->count);
-    int64_t c_off = 0, d_off = 0, r_off = 0, run_off = 0, body_off = 0;
+    int64_t c_off = 0, d_off = 0, r_off = 0, run_off = 0, body_off = 0, clean = 0, dirty = 0;
     for (int m = 0; m < b->count; ++m) {
         wmibm_handle *h = b->members[m];
         const wmibm_member_fields &fl = fields[m];
@@ -134,12 +138,21 @@ int upload_members(wmibm_batch *b, const wmibm_member_fields *fields, cudaStream
         mm.r_off = r_off;
         mm.run_off = run_off;
         mm.body_off = body_off;
+        direct_tile(mm, 16 / (int)sizeof(T), 0, 0, kDirectBatchLevels);
+        b->offsets.clean[m] = (int32_t)clean;
+        b->offsets.dirty[m] = (int32_t)dirty;
+        const int64_t tiles = (int64_t)mm.gx * mm.gy;
+        clean += tiles * ((mm.nz + mm.kc - 1) / mm.kc - mm.dcn);
+        dirty += tiles * mm.dcn;
         c_off += (int64_t)mm.nstrips * (mm.da + (mm.nz - mm.db));
         d_off += (int64_t)mm.nstrips * (mm.db - mm.da);
         r_off += mm.nb_w + mm.nb_uv;
         run_off += mm.nr_w + mm.nr_uv;
         body_off += mm.nbody_w + mm.nbody_uv;
     }
+    if (clean + dirty > INT32_MAX / 2) return berr(b, WMIBM_EINVAL, "the batch has too many nodes");
+    b->offsets.clean[b->count] = (int32_t)clean;
+    b->offsets.dirty[b->count] = (int32_t)dirty;
     b->clean_total = c_off;
     b->dirty_total = d_off;
     b->rec_total = r_off;
@@ -176,7 +189,13 @@ int step_impl(wmibm_batch *b, wmibm_band_stats *stats, int do_mask, cudaStream_t
     p.wait_ns = b->wait_ns;
     p.hold_release = b->hold_release;
     const int wall_blocks = 0;   // one wave of resident blocks
-    // untuned: two launches, the form the autotuner keeps on the measured ensembles
+    // untuned: the wall kernel, then the direct-load stencil
+    const wmibm_tuning none = {};
+    if (memcmp(&b->tuning, &none, sizeof(none)) == 0) {
+        int ds = batch_launch_direct<T, VEL>(b->members[0], (const Member<T> *)b->dev_members, b->count, p, b->cfg,
+                                             b->offsets, stream);
+        return ds ? berr(b, ds, "%s", b->members[0]->err) : WMIBM_OK;
+    }
     const int form = b->tuning.force_path == 0 ? 3 : b->tuning.force_path;
     int st = batch_launch<T, VEL>(b->members[0], (const Member<T> *)b->dev_members, b->count, p, b->cfg, b->max_nx,
                                   wall_blocks, form, stream);

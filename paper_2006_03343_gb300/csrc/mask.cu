@@ -59,10 +59,11 @@ int launch(wmibm_handle *h, void *u, void *v, void *w, const void *const gradp[3
 namespace wmibm {
 int wall_stress_impl(wmibm_handle *h, const void *u, const void *v, const void *w, void *const tau[6],
                      wmibm_band_stats *stats, cudaStream_t stream, const void *logz0);
-int force_impl(wmibm_handle *h, const void *const tau[6], void *fx, void *fy, void *fz, cudaStream_t stream, int bx,
-               int by, int kc);
-void force_default_tile(const wmibm_handle *h, int *bx, int *by, int *kc);
 int force_any(wmibm_handle *h, const void *const tau[6], void *fx, void *fy, void *fz, cudaStream_t stream);
+bool use_direct(const wmibm_handle *h, const void *const tau[6], void *const f[3], StencilConfig *c);
+int direct_stage(wmibm_handle *h, const void *const tau[6], const void *const own[6], void *const f[3], void *u,
+                 void *v, void *w, const void *const gradp[3], double dt, int do_mask, bool after, bool pdl,
+                 cudaStream_t stream, wmibm_band_stats *emit);
 bool stencil_config(const wmibm_handle *h, const void *const tau[6], void *const f[3], StencilConfig *out);
 int stencil_force_mask(wmibm_handle *h, void *u, void *v, void *w, const void *const tau[6], void *const f[3],
                        const void *const gradp[3], double dt, int do_mask, const StencilConfig &c, bool pdl,
@@ -74,36 +75,27 @@ int stencil_step_fused(wmibm_handle *h, void *u, void *v, void *w, void *const t
                        const void *const gradp[3], double dt, int do_mask, wmibm_band_stats *stats,
                        const StencilConfig &c, cudaStream_t stream);
 
-// Wall stress + force (+ mask) as two launches: the wall kernel, then the
-// pipelined stencil, which converts the wall launch's statistics (block 0); where
-// the pipeline does not take the grid, the wall kernel converts them itself and
-// the direct-load force (and mask) kernels follow.
+// Wall stress + force (+ mask) as two launches: the wall kernel, then the stencil,
+// which converts the wall launch's statistics and applies the mask.
 static int two_launch_step(wmibm_handle *h, const void *u, const void *v, const void *w, void *const tau[6],
                            void *fx, void *fy, void *fz, const void *const gradp[3], double dt, int do_mask,
                            wmibm_band_stats *stats, cudaStream_t stream)
 {
     void *const f[3] = {fx, fy, fz};
-    StencilConfig c;
-    if (stencil_config(h, (const void *const *)tau, f, &c)) {
-        int st = wall_model(h, u, v, w, tau, stats, h->logz0, stream, false);
-        if (st) return st;
-        return stencil_force_mask(h, const_cast<void *>(u), const_cast<void *>(v), const_cast<void *>(w),
-                                  (const void *const *)tau, f, gradp, dt, do_mask, c, true, stream, stats);
-    }
-    int st = wall_model(h, u, v, w, tau, stats, h->logz0, stream, true);
+    const void *const *in = (const void *const *)tau;
+    void *const uu = const_cast<void *>(u), *const vv = const_cast<void *>(v), *const ww = const_cast<void *>(w);
+    int st = wall_model(h, u, v, w, tau, stats, h->logz0, stream, false);
     if (st) return st;
-    st = force_any(h, (const void *const *)tau, fx, fy, fz, stream);
-    if (st || !do_mask) return st;
-    return mask_impl(h, const_cast<void *>(u), const_cast<void *>(v), const_cast<void *>(w), gradp, dt, stream);
+    StencilConfig c;
+    if (use_direct(h, in, f, &c))
+        return direct_stage(h, in, in, f, uu, vv, ww, gradp, dt, do_mask, true, true, stream, stats);
+    return stencil_force_mask(h, uu, vv, ww, in, f, gradp, dt, do_mask, c, true, stream, stats);
 }
 
 // Wall stress + force (+ mask) in one cooperative launch, where the tuning asks for
 // one and the pipelined stencil takes the grid; else *done stays 0 and nothing is
-// done.  Untuned handles take two launches: the stencil streams its clean units
-// beside the wall kernel's tail, and neither holds the other's registers (step in
-// us, one launch against two: 64^3 17.7 / 14.6, 192 x 96 x 96 26.9 / 23.1, cubes
-// 256 x 128 x 128 49.6 / 41.6, hill 512 x 256 x 256 237 / 228; FP64: 32^3 28.8 /
-// 28.3, 256 x 128 x 128 219 / 205).
+// done.  Untuned handles take two launches: the stencil streams its clean levels
+// beside the wall kernel's tail, and neither holds the other's registers.
 static int try_fused(wmibm_handle *h, void *u, void *v, void *w, void *const tau[6], void *fx, void *fy, void *fz,
                      const void *const gradp[3], double dt, int do_mask, wmibm_band_stats *stats,
                      cudaStream_t stream, int *done)
@@ -117,21 +109,16 @@ static int try_fused(wmibm_handle *h, void *u, void *v, void *w, void *const tau
     return stencil_step_fused(h, u, v, w, tau, f, gradp, dt, do_mask, stats, c, stream);
 }
 
-// force, then (do_mask) the body mask: one pipelined launch where the grid
-// allows, else the direct-load force kernel followed by the mask kernel.
+// force, then the body mask, in one launch.
 int force_mask_impl(wmibm_handle *h, void *u, void *v, void *w, void *const tau[6], void *fx, void *fy, void *fz,
-                    const void *const gradp[3], int do_mask, double dt, bool pdl, cudaStream_t stream)
+                    const void *const gradp[3], double dt, cudaStream_t stream)
 {
     void *const f[3] = {fx, fy, fz};
+    const void *const *in = (const void *const *)tau;
     StencilConfig c;
-    if (stencil_config(h, (const void *const *)tau, f, &c)) {
-        if (do_mask)
-            return stencil_force_mask(h, u, v, w, (const void *const *)tau, f, gradp, dt, 1, c, pdl, stream, nullptr);
-        return force_any(h, (const void *const *)tau, fx, fy, fz, stream);
-    }
-    int st = force_any(h, (const void *const *)tau, fx, fy, fz, stream);
-    if (st || !do_mask) return st;
-    return mask_impl(h, u, v, w, gradp, dt, stream);
+    if (use_direct(h, in, f, &c))
+        return direct_stage(h, in, in, f, u, v, w, gradp, dt, 1, true, false, stream, nullptr);
+    return stencil_force_mask(h, u, v, w, in, f, gradp, dt, 1, c, false, stream, nullptr);
 }
 
 int mask_impl(wmibm_handle *h, void *u, void *v, void *w, const void *const gradp[3], double dt, cudaStream_t stream)
@@ -191,8 +178,7 @@ extern "C" int wmibm_force_mask(wmibm_handle *h, const void *const tau[6], void 
     if (gradp && (!gradp[0] || !gradp[1] || !gradp[2]))
         return set_error(h, WMIBM_EINVAL, "gradp given with a NULL component");
     if (!isfinite(dt)) return set_error(h, WMIBM_EINVAL, "dt must be finite");
-    return force_mask_impl(h, u, v, w, const_cast<void *const *>(tau), fx, fy, fz, gradp, 1, dt, false,
-                           (cudaStream_t)stream);
+    return force_mask_impl(h, u, v, w, const_cast<void *const *>(tau), fx, fy, fz, gradp, dt, (cudaStream_t)stream);
 }
 
 extern "C" int wmibm_step(wmibm_handle *h, void *u, void *v, void *w, void *const tau[6], void *fx, void *fy,

@@ -18,6 +18,9 @@ struct Member {
     T cx, cy, cz;                 // 1/(2 dx), 1/(2 dy), 1/dz
     int32_t da, db;               // dirty levels [da, db)
     int64_t c_off, d_off;         // first index in the launch's clean / dirty unit spaces
+    // direct-load stencil: vectors per block row, rows per block, tiles along x and y, levels per
+    // chunk, and the chunks [dc0, dc0 + dcn) that hold dirty levels
+    int32_t bx, by, gx, gy, kc, dc0, dcn;
     const void *rec;              // band records (w-band first)
     int64_t nb_w, nb_uv, r_off;   // band counts; first index in the record space
     int64_t nzc_w, nzc_uv;        // band nodes whose sample point's level is clamped (reported in the stats)
@@ -35,6 +38,8 @@ template <typename T>
 struct KParams {
     Member<T> one;                // the member of a single-terrain launch (nmembers == 1)
     const Member<T> *list;        // device array of members (nmembers > 1)
+    // direct-load stencil: blocks of clean chunks, then of dirty ones, then those of the launch's tail
+    int32_t clean_blocks, dirty_blocks, tail_blocks;
     int nmembers;
     int64_t clean_total, dirty_total, rec_total, run_total, body_total;
     int stages, ncons;            // stages: depth of the ring of half A (half B has one more slot)
@@ -81,6 +86,14 @@ struct KParams {
     int hold_release;
 };
 
+constexpr int kMaxBatchMembers = 256;
+
+// First clean and first dirty block of each member of a batch, then the totals (a
+// kernel parameter: the look-up runs on the constant bank).
+struct DirectBatch {
+    int32_t clean[kMaxBatchMembers + 1], dirty[kMaxBatchMembers + 1];
+};
+
 template <typename T>
 void fill_member(const wmibm_handle *h, Member<T> &m, const void *const tau[6], void *const f[3], void *u, void *v,
                  void *w, const void *logz0, const void *const gradp[3], double dt, int rows);
@@ -91,6 +104,13 @@ int batch_launch(wmibm_handle *h0, const Member<T> *dev_members, int nmembers, c
 
 bool stencil_config(const wmibm_handle *h, const void *const tau[6], void *const f[3], StencilConfig *out);
 
-constexpr int kMaxBatchMembers = 256;
+// The direct-load stencil's tile of a member for vectors of v values: bx vectors by by rows, kc levels (0: chosen).
+template <typename T>
+void direct_tile(Member<T> &m, int v, int bx, int by, int kc);
+
+// The batch wall kernel, then the direct-load stencil over all members.
+template <typename T, typename VEL>
+int batch_launch_direct(wmibm_handle *h0, const Member<T> *dev_members, int nmembers, const KParams<T> &tmpl,
+                        const StencilConfig &c, const DirectBatch &offsets, cudaStream_t stream);
 
 }  // namespace wmibm

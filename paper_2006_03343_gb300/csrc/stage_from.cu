@@ -11,10 +11,9 @@ using namespace wmibm;
 namespace wmibm {
 int wall_model(wmibm_handle *h, const void *u, const void *v, const void *w, void *const tau[6],
                wmibm_band_stats *stats, const void *logz0, cudaStream_t stream, bool emit);
-int force_any(wmibm_handle *h, const void *const tau[6], void *fx, void *fy, void *fz, cudaStream_t stream);
-bool stencil_config(const wmibm_handle *h, const void *const tau[6], void *const f[3], StencilConfig *out);
-int stencil_force_from(wmibm_handle *h, const void *const tau[6], const void *const work[6], void *const f[3],
-                       const StencilConfig &c, cudaStream_t stream, wmibm_band_stats *emit);
+int direct_stage(wmibm_handle *h, const void *const tau[6], const void *const own[6], void *const f[3], void *u,
+                 void *v, void *w, const void *const gradp[3], double dt, int do_mask, bool after, bool pdl,
+                 cudaStream_t stream, wmibm_band_stats *emit);
 }  // namespace wmibm
 
 namespace {
@@ -44,23 +43,14 @@ __global__ void __launch_bounds__(kThreads) k_copy_levels(const __grid_constant_
     for (; q < n; q += stride) dst[q] = src[q];
 }
 
-// Levels [lo, hi) that the work buffer holds: with the pipelined stencil on the
-// caller's stresses those that dirty units read (their segments' first stage reads
-// the level below), else all.
-bool work_levels(const wmibm_handle *h, const void *const tau[6], void *const f[3], int32_t *lo, int32_t *hi,
-                 StencilConfig *c)
+// Levels [lo, hi) that the work buffer holds: those that the stencil reads for dirty
+// levels (the one below, and the one above, too).
+void work_levels(const wmibm_handle *h, int32_t *lo, int32_t *hi)
 {
-    const bool pipelined = stencil_config(h, tau, f, c);
-    if (!pipelined) {
-        *lo = 0;
-        *hi = h->nz;
-    } else if (h->dirty_hi <= h->dirty_lo) {
-        *lo = *hi = 0;
-    } else {
-        *lo = std::max(h->dirty_lo - 1, 0);
-        *hi = std::min(h->dirty_hi + 1, h->nz);
-    }
-    return pipelined;
+    *lo = *hi = 0;
+    if (h->dirty_hi <= h->dirty_lo) return;
+    *lo = std::max(h->dirty_lo - 1, 0);
+    *hi = std::min(h->dirty_hi + 1, h->nz);
 }
 
 // Bytes of one field of the work buffer, padded so that each field starts on a 16-byte boundary.
@@ -78,10 +68,8 @@ extern "C" int64_t wmibm_stage_work_bytes(const wmibm_handle *h, const void *con
     if (!h || !tau || !fx || !fy || !fz) return -1;
     for (int c = 0; c < 6; ++c)
         if (!tau[c]) return -1;
-    void *const f[3] = {const_cast<void *>(fx), const_cast<void *>(fy), const_cast<void *>(fz)};
     int32_t lo, hi;
-    StencilConfig c;
-    work_levels(h, tau, f, &lo, &hi, &c);
+    work_levels(h, &lo, &hi);
     return 6 * field_bytes(h, hi - lo);
 }
 
@@ -99,8 +87,7 @@ extern "C" int wmibm_wall_stress_force_from(wmibm_handle *h, const void *u, cons
     if (st) return st;
     void *const f[3] = {fx, fy, fz};
     int32_t lo, hi;
-    StencilConfig c;
-    const bool pipelined = work_levels(h, tau, f, &lo, &hi, &c);
+    work_levels(h, &lo, &hi);
     const int64_t field = field_bytes(h, hi - lo);
     if (work_bytes < 6 * field || (field > 0 && (!work || ((uintptr_t)work & 15u) != 0)))
         return set_error(h, WMIBM_EINVAL, "the work buffer must be 16-byte aligned and hold %lld bytes",
@@ -130,11 +117,8 @@ extern "C" int wmibm_wall_stress_force_from(wmibm_handle *h, const void *u, cons
         st = cuda_status(h, cudaGetLastError(), "k_copy_levels launch");
         if (st) return st;
     }
-    // without the pipeline on the caller's stresses (their alignment, say) the buffer holds them whole
-    if (!pipelined) {
-        st = wall_model(h, u, v, w, at, stats, h->logz0, s, true);
-        return st ? st : force_any(h, (const void *const *)at, fx, fy, fz, s);
-    }
     st = wall_model(h, u, v, w, at, stats, h->logz0, s, false);
-    return st ? st : stencil_force_from(h, tau, (const void *const *)at, f, c, s, stats);
+    if (st) return st;
+    return direct_stage(h, tau, (const void *const *)at, f, nullptr, nullptr, nullptr, nullptr, 0.0, 0, true, true, s,
+                        stats);
 }

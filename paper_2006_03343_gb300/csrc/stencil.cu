@@ -34,6 +34,7 @@
 // Every mbarrier wait is bounded: on time-out the kernel records a status code
 // in device memory and leaves its loops.
 #include <algorithm>
+#include <type_traits>
 
 #include "band.cuh"
 #include "members.cuh"
@@ -574,6 +575,17 @@ __device__ void produce(const KParams<T> &p, T *ring_a, T *ring_b, uint64_t *ful
     }
 }
 
+// -(dx cx + dy cy + dz cz), the differences of one component of -div(tau): rounded
+// alike in every form of the stencil.
+__device__ __forceinline__ float divergence(float dx, float cx, float dy, float cy, float dz, float cz)
+{
+    return -fmaf(dz, cz, fmaf(dy, cy, dx * cx));
+}
+__device__ __forceinline__ double divergence(double dx, double cx, double dy, double cy, double dz, double cz)
+{
+    return -fma(dz, cz, fma(dy, cy, dx * cx));
+}
+
 // ------------------------------------------------------------------------- //
 // consumers: f for the TY rows of a main stage
 // ------------------------------------------------------------------------- //
@@ -641,7 +653,7 @@ __device__ void consume_level(const ConsView<T> &cv, int ncons, const T *cur, co
 #pragma unroll
             for (int e = 0; e < V; ++e) {
                 const T xxm_ = e == 0 ? xxl : xx.v[e - 1], xxp_ = e == V - 1 ? xxr : xx.v[e + 1];
-                Fx.v[e] = -((xxp_ - xxm_) * cx + (xyp.v[e] - xym.v[e]) * cy + (xz1.v[e] - xz0.v[e]) * cz);
+                Fx.v[e] = divergence(xxp_ - xxm_, cx, xyp.v[e] - xym.v[e], cy, xz1.v[e] - xz0.v[e], cz);
             }
             if (valid) stg(cv.f[0] + o, Fx);
         }
@@ -657,7 +669,7 @@ __device__ void consume_level(const ConsView<T> &cv, int ncons, const T *cur, co
 #pragma unroll
             for (int e = 0; e < V; ++e) {
                 const T xym_ = e == 0 ? xyl : xy.v[e - 1], xyp_ = e == V - 1 ? xyr : xy.v[e + 1];
-                Fy.v[e] = -((xyp_ - xym_) * cx + (yyp.v[e] - yym.v[e]) * cy + (yz1.v[e] - yz0.v[e]) * cz);
+                Fy.v[e] = divergence(xyp_ - xym_, cx, yyp.v[e] - yym.v[e], cy, yz1.v[e] - yz0.v[e], cz);
             }
             if (valid) stg(cv.f[1] + o, Fy);
         }
@@ -677,7 +689,7 @@ __device__ void consume_level(const ConsView<T> &cv, int ncons, const T *cur, co
 #pragma unroll
             for (int e = 0; e < V; ++e) {
                 const T xzm_ = e == 0 ? xzl : xz0.v[e - 1], xzp_ = e == V - 1 ? xzr : xz0.v[e + 1];
-                const T fz = -((xzp_ - xzm_) * cx + (yz0p.v[e] - yz0m.v[e]) * cy + (zz.v[e] - zzm.v[e]) * cz);
+                const T fz = divergence(xzp_ - xzm_, cx, yz0p.v[e] - yz0m.v[e], cy, zz.v[e] - zzm.v[e], cz);
                 Fz.v[e] = bottom ? T(0) : fz;
             }
             if (valid) stg(cv.f[2] + o, Fz);
@@ -1686,6 +1698,192 @@ __global__ void __launch_bounds__(512) k_stencil(KParams<T> p)
     }
 }
 
+// ------------------------------------------------------------------------- //
+// direct-load stencil
+// ------------------------------------------------------------------------- //
+template <typename T, int V>
+struct Vec {
+    T v[V];
+};
+__device__ __forceinline__ Vec<float, 4> ldv(const float *p, Vec<float, 4> *)
+{
+    const float4 a = *reinterpret_cast<const float4 *>(p);
+    return Vec<float, 4>{{a.x, a.y, a.z, a.w}};
+}
+__device__ __forceinline__ Vec<float, 2> ldv(const float *p, Vec<float, 2> *)
+{
+    const float2 a = *reinterpret_cast<const float2 *>(p);
+    return Vec<float, 2>{{a.x, a.y}};
+}
+__device__ __forceinline__ Vec<double, 2> ldv(const double *p, Vec<double, 2> *)
+{
+    const double2 a = *reinterpret_cast<const double2 *>(p);
+    return Vec<double, 2>{{a.x, a.y}};
+}
+template <typename T>
+__device__ __forceinline__ Vec<T, 1> ldv(const T *p, Vec<T, 1> *)
+{
+    return Vec<T, 1>{{*p}};
+}
+__device__ __forceinline__ void stv(float *p, const Vec<float, 4> &x)
+{
+    *reinterpret_cast<float4 *>(p) = make_float4(x.v[0], x.v[1], x.v[2], x.v[3]);
+}
+__device__ __forceinline__ void stv(float *p, const Vec<float, 2> &x)
+{
+    *reinterpret_cast<float2 *>(p) = make_float2(x.v[0], x.v[1]);
+}
+__device__ __forceinline__ void stv(double *p, const Vec<double, 2> &x)
+{
+    *reinterpret_cast<double2 *>(p) = make_double2(x.v[0], x.v[1]);
+}
+template <typename T>
+__device__ __forceinline__ void stv(T *p, const Vec<T, 1> &x)
+{
+    *p = x.v[0];
+}
+
+// What a thread loads for level k: the vectors of its row and of the rows beside it,
+// the values beyond the vector's ends, txz and tyz of the level above.
+template <typename T, int V>
+struct Level {
+    Vec<T, V> xx, xy, xyjm, xyjp, yyjm, yyjp, yzjm, yzjp, zz, xz_kp, yz_kp;
+    T xxl, xxr, xyl, xyr, xzl, xzr;
+};
+
+constexpr int kDirectThreads = 256;
+// Resident blocks per SM that the registers are held to.
+template <typename T, int V>
+constexpr int kDirectBlocks = sizeof(T) == 4 && V <= 2 ? 4 : 3;
+
+struct NoBatch {
+};
+
+// f = -div(tau) with loads through L1 (periodic central differences, Eqs. 15-16 in
+// z), the stencil of untuned launches.  A thread owns V consecutive x-points of one
+// row and marches up a chunk of kc levels, carrying txz, tyz (level k+1 -> k) and tzz
+// (k -> k-1) in registers; the x-neighbours at the vector's ends and the rows beside
+// it are the neighbouring threads' lines, so DRAM sees each array once.  Bound by
+// HBM: many small blocks keep more loads in flight than the bulk-copy pipeline's
+// stages, and blocks that are resident together are neighbours in y, so that the
+// edge rows that the pipeline's strips read twice come from L2.  All of a level's
+// loads go out before the first is used, with 32-bit offsets from the array bases.
+// Chunks of two levels: as fast as any (the levels below and above a chunk come from
+// L2) and the finest grain for the launch's end.
+// Force alone (one GB300, FP32, this / the pipeline): hill 512 x 256 x 256 171 / 218
+// us (7.06 TB/s), cubes 256 x 128 x 128 27.0 / 31.0, 192 x 96 x 96 14.6 / 18.0; FP64
+// 256 x 128 x 128, bound by its arithmetic, 174 / 180.
+//
+// After a wall launch (AFTER) the grid is a programmatic dependent of it: blocks of
+// clean chunks come first and start at once, those of dirty chunks wait for the wall
+// kernel, and the tail's blocks apply the body mask (Eq. 27) and convert the
+// statistics after the same wait.  BATCH: the blocks of all members, clean ones
+// first.  Loads are not of the read-only kind: an SM's cache may hold what a clean
+// block read of a sector that a dirty level's first row shares.
+template <typename T, typename VEL, int V, bool AFTER, typename Batch>
+__global__ void __launch_bounds__(kDirectThreads, (kDirectBlocks<T, V>))
+    k_direct(const __grid_constant__ KParams<T> p, const __grid_constant__ Batch batch)
+{
+    constexpr bool BATCH = !std::is_same<Batch, NoBatch>::value;
+    using W = Vec<T, V>;
+    int b = blockIdx.x;
+    const int t = threadIdx.x;
+    if (AFTER && b >= p.clean_blocks + p.dirty_blocks) {
+        b -= p.clean_blocks + p.dirty_blocks;
+        wait_wall_kernel();
+        if (p.do_mask)
+            mask_phase<T, VEL>(p, (int64_t)b * kDirectThreads + t, (int64_t)p.tail_blocks * kDirectThreads);
+        if (!BATCH && p.emit_stats && b == 0 && t == 0)
+            stats_emit(p.sacc, p.stats, p.one.nb_w, p.one.nb_uv, p.one.nzc_w, p.one.nzc_uv);
+        return;
+    }
+    const bool dirty = AFTER && b >= p.clean_blocks;
+    if (dirty) b -= p.clean_blocks;
+    const Member<T> *mm = &p.one;
+    if constexpr (BATCH) {
+        const int32_t *first = dirty ? batch.dirty : batch.clean;
+        int lo = 0, hi = p.nmembers - 1;
+        while (lo < hi) {
+            const int mid = (lo + hi + 1) >> 1;
+            if (first[mid] <= b) lo = mid;
+            else hi = mid - 1;
+        }
+        b -= first[lo];
+        mm = p.list + lo;
+    }
+    const Member<T> &m = *mm;
+    const int nx = m.nx, ny = m.ny, nz = m.nz, bx = m.bx, gx = m.gx, kc = m.kc;
+    const int tiles = gx * m.gy;
+    int c = b / tiles;
+    const int tile = b - c * tiles, tile_y = tile / gx, tile_x = tile - tile_y * gx;
+    if (dirty) c += m.dc0;
+    else if (c >= m.dc0) c += m.dcn;
+    const int ly = t / bx, by = m.by;
+    const int i = (tile_x * bx + (t - ly * bx)) * V, j = tile_y * by + ly;
+    // what follows this launch in the stream relies on the wall kernel's end as well
+    if (AFTER && (dirty || blockIdx.x == gridDim.x - 1)) {
+        wait_wall_kernel();
+        __threadfence();
+    }
+    if (ly >= by || i >= nx || j >= ny) return;
+    const int k0 = c * kc, k1 = min(k0 + kc, nz), plane = nx * ny;
+    const int im = (i == 0) ? nx - 1 : i - 1, ip = (i + V == nx) ? 0 : i + V;
+    const int jm = (j == 0) ? ny - 1 : j - 1, jp = (j + 1 == ny) ? 0 : j + 1;
+    const int at = j * nx + i, atm = jm * nx + i, atp = jp * nx + i, left = j * nx + im, right = j * nx + ip;
+    const T cx = m.cx, cy = m.cy, cz = m.cz;
+    T *const fx = m.f[0], *const fy = m.f[1], *const fz = m.f[2];
+    auto field = [&](int a, bool own) -> const T * { return (BATCH || own) ? m.tau[a] : m.tin[a]; };
+    const bool own0 = k0 >= m.da && k0 < m.db;
+    W xz_k = ldv(field(4, own0) + k0 * plane + at, (W *)nullptr);
+    W yz_k = ldv(field(5, own0) + k0 * plane + at, (W *)nullptr);
+    W zz_km;
+    for (int e = 0; e < V; ++e) zz_km.v[e] = T(0);
+    if (k0 > 0) zz_km = ldv(field(3, own0) + (k0 - 1) * plane + at, (W *)nullptr);
+    for (int k = k0; k < k1; ++k) {
+        const bool own = k >= m.da && k < m.db, top = k == nz - 1;
+        const int o = k * plane, up = top ? o : o + plane;
+        const T *const txx = field(0, own) + o, *const txy = field(1, own) + o, *const tyy = field(2, own) + o;
+        const T *const tzz = field(3, own) + o, *const txz = field(4, own), *const tyz = field(5, own);
+        Level<T, V> l;
+        l.xx = ldv(txx + at, (W *)nullptr);
+        l.xxl = txx[left];
+        l.xxr = txx[right];
+        l.xy = ldv(txy + at, (W *)nullptr);
+        l.xyl = txy[left];
+        l.xyr = txy[right];
+        l.xyjm = ldv(txy + atm, (W *)nullptr);
+        l.xyjp = ldv(txy + atp, (W *)nullptr);
+        l.yyjm = ldv(tyy + atm, (W *)nullptr);
+        l.yyjp = ldv(tyy + atp, (W *)nullptr);
+        l.yzjm = ldv(tyz + o + atm, (W *)nullptr);
+        l.yzjp = ldv(tyz + o + atp, (W *)nullptr);
+        l.xzl = txz[o + left];
+        l.xzr = txz[o + right];
+        l.zz = ldv(tzz + at, (W *)nullptr);
+        l.xz_kp = ldv(txz + up + at, (W *)nullptr);
+        l.yz_kp = ldv(tyz + up + at, (W *)nullptr);
+        W Fx, Fy, Fz;
+#pragma unroll
+        for (int e = 0; e < V; ++e) {
+            const T xxm = e == 0 ? l.xxl : l.xx.v[e - 1], xxp = e == V - 1 ? l.xxr : l.xx.v[e + 1];
+            const T xym = e == 0 ? l.xyl : l.xy.v[e - 1], xyp = e == V - 1 ? l.xyr : l.xy.v[e + 1];
+            const T xzm = e == 0 ? l.xzl : xz_k.v[e - 1], xzp = e == V - 1 ? l.xzr : xz_k.v[e + 1];
+            const T vx = divergence(xxp - xxm, cx, l.xyjp.v[e] - l.xyjm.v[e], cy, l.xz_kp.v[e] - xz_k.v[e], cz);
+            const T vy = divergence(xyp - xym, cx, l.yyjp.v[e] - l.yyjm.v[e], cy, l.yz_kp.v[e] - yz_k.v[e], cz);
+            const T vz = divergence(xzp - xzm, cx, l.yzjp.v[e] - l.yzjm.v[e], cy, l.zz.v[e] - zz_km.v[e], cz);
+            Fx.v[e] = top ? T(0) : vx;
+            Fy.v[e] = top ? T(0) : vy;
+            Fz.v[e] = (top || k == 0) ? T(0) : vz;
+        }
+        stv(fx + o + at, Fx);
+        stv(fy + o + at, Fy);
+        stv(fz + o + at, Fz);
+        xz_k = l.xz_kp;
+        yz_k = l.yz_kp;
+        zz_km = l.zz;
+    }
+}
+
 constexpr int kMaxDynSmem = 200 * 1024;
 
 template <typename T, typename VEL, int TY, int MODE>
@@ -1885,9 +2083,119 @@ int launch_wall_single(wmibm_handle *h, void *const tau[6], const void *u, const
     return cuda_status(h, cudaGetLastError(), "k_wall launch");
 }
 
+// The direct-load stencil over p's member(s): its grid, then the launch.  body_total,
+// do_mask and emit_stats are the tail's work; pdl: the wall kernel comes just before.
+template <typename T, typename VEL, int V, bool AFTER, typename Batch>
+int launch_direct(wmibm_handle *h, KParams<T> &p, const Batch &batch, bool pdl, cudaStream_t stream)
+{
+    const int64_t want = (p.body_total + 2 * kDirectThreads - 1) / (2 * kDirectThreads);
+    p.tail_blocks = p.do_mask ? (int32_t)std::min<int64_t>(want, 4 * (int64_t)h->sm_count) : 0;
+    if (p.emit_stats && p.tail_blocks == 0) p.tail_blocks = 1;
+    if (!AFTER) p.tail_blocks = 0;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)(p.clean_blocks + p.dirty_blocks + p.tail_blocks));
+    cfg.blockDim = dim3(kDirectThreads);
+    cfg.stream = stream;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = AFTER && pdl ? 1 : 0;
+    return cuda_status(h, cudaLaunchKernelEx(&cfg, k_direct<T, VEL, V, AFTER, Batch>, p, batch), "k_direct launch");
+}
+
+// Values per vector that every row of these arrays is aligned for.
+template <typename T>
+int direct_vector(const Member<T> &m)
+{
+    for (int v = 16 / (int)sizeof(T); v > 1; v /= 2) {
+        const uintptr_t mask = v * sizeof(T) - 1;
+        bool fits = m.nx % v == 0;
+        for (int a = 0; a < 6; ++a) fits = fits && ((uintptr_t)m.tau[a] & mask) == 0 && ((uintptr_t)m.tin[a] & mask) == 0;
+        for (int a = 0; a < 3; ++a) fits = fits && ((uintptr_t)m.f[a] & mask) == 0;
+        if (fits) return v;
+    }
+    return 1;
+}
+
+template <typename T, typename VEL, bool AFTER>
+int direct_single(wmibm_handle *h, KParams<T> &p, bool pdl, cudaStream_t stream)
+{
+    const int v = direct_vector(p.one);
+    direct_tile(p.one, v, h->tuning.direct_bx, h->tuning.direct_by, h->tuning.direct_kc);
+    const int64_t tiles = (int64_t)p.one.gx * p.one.gy, chunks = (p.one.nz + p.one.kc - 1) / p.one.kc;
+    if (tiles * chunks > INT32_MAX / 2) return set_error(h, WMIBM_EINVAL, "grid too large for the force launch");
+    p.clean_blocks = (int32_t)(tiles * (chunks - p.one.dcn));
+    p.dirty_blocks = (int32_t)(tiles * p.one.dcn);
+    if constexpr (sizeof(T) == 4) {
+        if (v == 4) return launch_direct<T, VEL, 4, AFTER>(h, p, NoBatch{}, pdl, stream);
+    }
+    if (v == 2) return launch_direct<T, VEL, 2, AFTER>(h, p, NoBatch{}, pdl, stream);
+    return launch_direct<T, VEL, 1, AFTER>(h, p, NoBatch{}, pdl, stream);
+}
+
+template <typename T, typename VEL>
+int direct_impl(wmibm_handle *h, const void *const tau[6], const void *const own[6], void *const f[3], void *u,
+                void *v, void *w, const void *const gradp[3], double dt, int do_mask, bool after, bool pdl,
+                cudaStream_t stream, wmibm_band_stats *emit)
+{
+    KParams<T> p;
+    fill_member<T>(h, p.one, own, f, u, v, w, nullptr, gradp, dt, 0);
+    for (int a = 0; a < 6; ++a) p.one.tin[a] = (const T *)tau[a];
+    single_params<T>(h, p, after);
+    p.do_mask = do_mask;
+    p.stats = emit;
+    p.emit_stats = emit != nullptr;
+    if (after) return direct_single<T, VEL, true>(h, p, pdl, stream);
+    return direct_single<T, T, false>(h, p, false, stream);      // no mask: the velocity's type does not matter
+}
+
 }  // namespace
 
 namespace wmibm {
+
+template <typename T>
+void direct_tile(Member<T> &m, int v, int bx, int by, int kc)
+{
+    const int nq = m.nx / v, across = (nq + 31) / 32;
+    // blocks of equal width, at most a warp unless the tuning says otherwise
+    m.bx = bx > 0 ? std::min(std::min(bx, nq), kDirectThreads) : (nq + across - 1) / across;
+    m.kc = kc > 0 ? kc : 2;
+    m.by = kDirectThreads / m.bx;
+    if (by > 0) m.by = std::min(by, m.by);
+    m.gx = (nq + m.bx - 1) / m.bx;
+    m.gy = (m.ny + m.by - 1) / m.by;
+    m.dc0 = m.da / m.kc;
+    m.dcn = m.db > m.da ? (m.db + m.kc - 1) / m.kc - m.dc0 : 0;
+}
+template void direct_tile<float>(Member<float> &, int, int, int, int);
+template void direct_tile<double>(Member<double> &, int, int, int, int);
+
+// Whether this handle's stencil is the direct-load one: untuned, or asked for
+// (force_path 2), or on rows that the pipeline does not take.
+bool use_direct(const wmibm_handle *h, const void *const tau[6], void *const f[3], StencilConfig *c)
+{
+    const wmibm_tuning &t = h->tuning;
+    if (t.force_path == 2) return true;
+    if (t.force_path == 0 && t.rows == 0 && t.stages == 0 && t.consumer_warps == 0 && t.blocks_per_sm == 0 &&
+        t.dyn_chunk == 0)
+        return true;
+    return !stencil_config(h, tau, f, c);
+}
+
+// The direct-load stencil.  own: the stresses that dirty levels are read from (tau
+// itself, or a work buffer).  after: dirty levels and the body mask wait for the
+// kernel before, the wall kernel when pdl is set; emit: its statistics, or NULL.
+int direct_stage(wmibm_handle *h, const void *const tau[6], const void *const own[6], void *const f[3], void *u,
+                 void *v, void *w, const void *const gradp[3], double dt, int do_mask, bool after, bool pdl,
+                 cudaStream_t stream, wmibm_band_stats *emit)
+{
+    if (h->dtype == WMIBM_F64)
+        return direct_impl<double, double>(h, tau, own, f, u, v, w, gradp, dt, do_mask, after, pdl, stream, emit);
+    if (h->vel_dtype == WMIBM_BF16 && do_mask)
+        return direct_impl<float, __nv_bfloat16>(h, tau, own, f, u, v, w, gradp, dt, do_mask, after, pdl, stream, emit);
+    return direct_impl<float, float>(h, tau, own, f, u, v, w, gradp, dt, do_mask, after, pdl, stream, emit);
+}
 
 // Fills the member descriptor of handle h with the given fields.
 template <typename T>
@@ -2044,33 +2352,6 @@ int stencil_force_mask(wmibm_handle *h, void *u, void *v, void *w, const void *c
     return launch_stencil<float, float, kAfterWall>(h, p, c, stream, pdl, h->nx);
 }
 
-// The pipelined stencil after a wall launch on `work`, which holds the levels that
-// dirty units read; clean units read the caller's stresses.
-int stencil_force_from(wmibm_handle *h, const void *const tau[6], const void *const work[6], void *const f[3],
-                       const StencilConfig &c, cudaStream_t stream, wmibm_band_stats *emit)
-{
-    if (h->dtype == WMIBM_F64) {
-        KParams<double> p;
-        fill_member<double>(h, p.one, work, f, nullptr, nullptr, nullptr, nullptr, nullptr, 0.0, c.rows);
-        for (int a = 0; a < 6; ++a) p.one.tin[a] = (const double *)tau[a];
-        single_params<double>(h, p, true);
-        p.stages = c.stages;
-        p.ncons = c.consumer_warps;
-        p.stats = emit;
-        p.emit_stats = emit != nullptr;
-        return launch_stencil<double, double, kAfterWall>(h, p, c, stream, true, h->nx);
-    }
-    KParams<float> p;
-    fill_member<float>(h, p.one, work, f, nullptr, nullptr, nullptr, nullptr, nullptr, 0.0, c.rows);
-    for (int a = 0; a < 6; ++a) p.one.tin[a] = (const float *)tau[a];
-    single_params<float>(h, p, true);
-    p.stages = c.stages;
-    p.ncons = c.consumer_warps;
-    p.stats = emit;
-    p.emit_stats = emit != nullptr;
-    return launch_stencil<float, float, kAfterWall>(h, p, c, stream, true, h->nx);
-}
-
 template <typename T, typename VEL>
 int step_fused_impl(wmibm_handle *h, void *u, void *v, void *w, void *const tau[6], void *const f[3],
                     const void *const gradp[3], double dt, int do_mask, wmibm_band_stats *stats,
@@ -2166,26 +2447,15 @@ int wall_model_with_scratch(wmibm_handle *h, const void *u, const void *v, const
                                             stream);
 }
 
-// One batched step: the batch wall kernel, then the batch stencil (force + mask)
-// as its programmatic dependent (form 3); or one cooperative launch of the batch
-// stencil with every member's band records as wall stages of its blocks (form 5)
-// or in wall warps beside its producer and consumers (form 6).
-// tmpl carries the launch-wide fields.
+// The batch wall kernel over p's members.
 template <typename T, typename VEL>
-int batch_launch(wmibm_handle *h0, const Member<T> *dev_members, int nmembers, const KParams<T> &tmpl,
-                 const StencilConfig &c, int max_nx, int wall_blocks, int form, cudaStream_t stream)
+static int launch_wall_batch(wmibm_handle *h0, const KParams<T> &p, const StencilConfig &c, int wall_blocks,
+                             cudaStream_t stream)
 {
-    KParams<T> p = tmpl;
-    p.list = dev_members;
-    p.nmembers = nmembers;
-    p.stages = c.stages;
-    p.ncons = c.consumer_warps;
-    if (form == 5) return launch_stencil_ty<T, VEL, 0, kInterleaved>(h0, p, c, stream, false, max_nx);
-    if (form == 6) return launch_stencil_ty<T, VEL, 0, kWarpSpec>(h0, p, c, stream, false, max_nx);
     // two chunks of 2 x 256 records in shared memory, then the member table
     // (3 offsets and 3 pointers a member, 8 bytes each, and two end entries)
     const size_t chunks = 2 * 2 * 256 * sizeof(typename RecOf<T>::type);
-    const size_t wsmem = chunks + (size_t)(6 * nmembers + 2) * 8;
+    const size_t wsmem = chunks + (size_t)(6 * p.nmembers + 2) * 8;
     const size_t wsmem_max = chunks + (size_t)(6 * kMaxBatchMembers + 2) * 8;
     static int per_sm = 0;                 // once per instantiation and process (at the largest table)
     if (per_sm == 0) {
@@ -2202,10 +2472,54 @@ int batch_launch(wmibm_handle *h0, const Member<T> *dev_members, int nmembers, c
         wall_blocks = bps * h0->sm_count;
     }
     k_wall_batch<T, VEL><<<(unsigned)wall_blocks, 256, wsmem, stream>>>(p);
-    int st = cuda_status(h0, cudaGetLastError(), "k_wall_batch launch");
+    return cuda_status(h0, cudaGetLastError(), "k_wall_batch launch");
+}
+
+// One batched step: the batch wall kernel, then the batch stencil (force + mask)
+// as its programmatic dependent (form 3); or one cooperative launch of the batch
+// stencil with every member's band records as wall stages of its blocks (form 5)
+// or in wall warps beside its producer and consumers (form 6).
+// tmpl carries the launch-wide fields.
+template <typename T, typename VEL>
+int batch_launch(wmibm_handle *h0, const Member<T> *dev_members, int nmembers, const KParams<T> &tmpl,
+                 const StencilConfig &c, int max_nx, int wall_blocks, int form, cudaStream_t stream)
+{
+    KParams<T> p = tmpl;
+    p.list = dev_members;
+    p.nmembers = nmembers;
+    p.stages = c.stages;
+    p.ncons = c.consumer_warps;
+    if (form == 5) return launch_stencil_ty<T, VEL, 0, kInterleaved>(h0, p, c, stream, false, max_nx);
+    if (form == 6) return launch_stencil_ty<T, VEL, 0, kWarpSpec>(h0, p, c, stream, false, max_nx);
+    int st = launch_wall_batch<T, VEL>(h0, p, c, wall_blocks, stream);
     if (st) return st;
     return launch_stencil_ty<T, VEL, 0, kAfterWall>(h0, p, c, stream, true, max_nx);
 }
+
+template <typename T, typename VEL>
+int batch_launch_direct(wmibm_handle *h0, const Member<T> *dev_members, int nmembers, const KParams<T> &tmpl,
+                        const StencilConfig &c, const DirectBatch &offsets, cudaStream_t stream)
+{
+    KParams<T> p = tmpl;
+    p.list = dev_members;
+    p.nmembers = nmembers;
+    p.clean_blocks = offsets.clean[nmembers];
+    p.dirty_blocks = offsets.dirty[nmembers];
+    p.emit_stats = 0;                       // the batch wall kernel converts the statistics
+    int st = launch_wall_batch<T, VEL>(h0, p, c, 0, stream);
+    if (st) return st;
+    constexpr int V = 16 / (int)sizeof(T);
+    if (nmembers == 1) return launch_direct<T, VEL, V, true>(h0, p, NoBatch{}, true, stream);
+    return launch_direct<T, VEL, V, true>(h0, p, offsets, true, stream);
+}
+
+template int batch_launch_direct<float, float>(wmibm_handle *, const Member<float> *, int, const KParams<float> &,
+                                               const StencilConfig &, const DirectBatch &, cudaStream_t);
+template int batch_launch_direct<float, __nv_bfloat16>(wmibm_handle *, const Member<float> *, int,
+                                                       const KParams<float> &, const StencilConfig &,
+                                                       const DirectBatch &, cudaStream_t);
+template int batch_launch_direct<double, double>(wmibm_handle *, const Member<double> *, int, const KParams<double> &,
+                                                 const StencilConfig &, const DirectBatch &, cudaStream_t);
 
 template int batch_launch<float, float>(wmibm_handle *, const Member<float> *, int, const KParams<float> &,
                                         const StencilConfig &, int, int, int, cudaStream_t);
