@@ -123,7 +123,7 @@ def profiled_batch_traffic(form, dtype, points):
     summary of that form (taken on fewer members: the bytes per node carry over,
     the members being drawn the same way), if it was taken on the current kernel
     sources (else None)."""
-    name = {3: "batch_two_launch", 5: "batch_interleaved", 6: "batch_wall_warps"}[form]
+    name = {0: "batch_direct", 3: "batch_two_launch", 5: "batch_interleaved", 6: "batch_wall_warps"}[form]
     path = os.path.join(ROOT, "profiles", f"{name}_ensemble_{dtype}.md")
     try:
         text = open(path).read()
@@ -594,13 +594,15 @@ def run_ours(args):
     # phase inside (one-launch form), or the force stencil (two-launch form)
     step_bytes = h.traffic_bytes(4)          # wall-model bytes + 36 B/pt (FP32) of the force stream
     peak, peak_kind = measured_peak()
-    one_launch = h.get_tuning().force_path != 3
+    one_launch = h.get_tuning().force_path not in (0, 2, 3)
     if one_launch:
         kernel, kbytes, kms = "stencil_fused", step_bytes, float(np.mean(step_ms))
         kdesc = "k_stencil<fused> (wall phase + pipelined force, one cooperative launch)"
     else:
         kernel, kbytes, kms = "stencil_force", h.traffic_bytes(1), float(np.mean(parts["force"]))
-        kdesc = "k_stencil (pipelined force; the wall model is a kernel of its own)"
+        kdesc = ("k_stencil (pipelined force; the wall model is a kernel of its own)"
+                 if h.get_tuning().force_path == 3 else
+                 "k_direct (direct-load force; the wall model is a kernel of its own)")
     achieved = kbytes / (kms * 1e-3) / 1e9
     traffic = profiled_traffic(kernel, args.workload, args.dtype, args.vel_dtype)
 
@@ -795,7 +797,8 @@ def accuracy_report(gpu_tau, gpu_f, ref):
     return out
 
 
-ENSEMBLE_FORMS = {3: "two launches: the batch wall kernel, then the batch stencil as its programmatic dependent",
+ENSEMBLE_FORMS = {0: "two launches: the batch wall kernel, then the direct-load stencil as its programmatic dependent",
+                  3: "two launches: the batch wall kernel, then the batch stencil as its programmatic dependent",
                   5: "one cooperative launch: the batch stencil with every member's band records as interleaved "
                      "wall stages",
                   6: "one cooperative launch: the batch stencil with wall warps beside its producer and consumer "
@@ -872,8 +875,8 @@ def run_ensemble(args):
         tuned = {"tuning": {}, "default": True}
     else:
         tuned = autotune.tune_batch(batch, stats)
-    form = batch.get_tuning().get("force_path", 0)
-    form = 3 if form == 0 else form          # an untuned batch takes two launches
+    fields_set = {k: v for k, v in batch.get_tuning().items() if v}
+    form = fields_set.get("force_path", 3) if fields_set else 0     # an untuned batch takes the direct-load stencil
     for _ in range(max(args.warmup, 3)):
         flush.zero_()
         batch.wall_stress_force(stats)
@@ -1120,7 +1123,7 @@ def run_ensemble(args):
                            "how": "the members' wall stress + force one after the other, in one CUDA graph"}
             if extras else None,
             "timing": "per step: CUDA events around one graph replay of the batch wall stress + force",
-            "gpu_launches": args.steps * (2 if form == 3 else 1), "device_status": status,
+            "gpu_launches": args.steps * (2 if form in (0, 3) else 1), "device_status": status,
             "accuracy": accuracy, "f64_form": f64_form, "clocks": clocks, "e2e": e2e, "cpu_baseline": cpu}
     if world > 1:
         line["config"]["parallelism"] = f"{world} ranks, one GPU each, every rank its own copy of the ensemble"

@@ -259,11 +259,11 @@ int wmibm_mask(wmibm_handle *h, void *u, void *v, void *w, const void *const gra
 /*
  * wmibm_step - wmibm_wall_stress, wmibm_force and wmibm_mask in that order on
  * one stream: one pass of the whole per-step stress stage, with the same results
- * as the three calls.  By default (tuning.force_path 0 or 3) it is two launches
- * where the pipelined stencil takes the grid (see wmibm_force_mask): the
- * wall-model kernel, then the force + mask kernel as its programmatic dependent,
- * which streams the stages that read no band or solid node meanwhile.  With
- * force_path 1, 4, 5 or 6 it is ONE cooperative launch there: in every block the
+ * as the three calls.  By default it is two launches: the wall-model kernel, then
+ * the force + mask kernel (direct loads) as its programmatic dependent, whose blocks
+ * on levels that read no band or solid node start meanwhile; with force_path 3 the
+ * second is the pipelined kernel where it takes the grid (see wmibm_force_mask).
+ * With force_path 1, 4, 5 or 6 it is ONE cooperative launch there: in every block the
  * consumer warps (1) first evaluate the block's share of the band nodes and solid
  * runs while the producer streams the clean stages; stages that read them wait
  * (bounded) until every block has finished its wall share; the body mask follows
@@ -303,12 +303,11 @@ int64_t wmibm_stage_work_bytes(const wmibm_handle *h, const void *const tau[6], 
                                const void *fz);
 
 /*
- * wmibm_force_mask - wmibm_force followed by wmibm_mask, in one launch where the
- * grid allows the pipelined stencil (nx a multiple of 4 for F32 or 2 for F64,
- * ny >= 3, 16-byte aligned stress and force buffers, full x-rows that fit the
- * shared-memory stages): the kernel forms f and then applies Eq. 27 to u, v, w.
- * Otherwise the force and mask kernels run back to back.  Arguments as in
- * wmibm_force and wmibm_mask.
+ * wmibm_force_mask - wmibm_force followed by wmibm_mask, in one launch: the kernel
+ * forms f and applies Eq. 27 to u, v, w.  Arguments as in wmibm_force and wmibm_mask.
+ * The pipelined stencil, which tuning can ask for, takes grids with nx a multiple of
+ * 4 for F32 or 2 for F64, ny >= 3, 16-byte aligned stress and force buffers and full
+ * x-rows that fit its shared-memory stages; on others the direct-load kernel runs.
  */
 int wmibm_force_mask(wmibm_handle *h, const void *const tau[6], void *fx, void *fy, void *fz, void *u, void *v,
                      void *w, const void *const gradp[3], double dt, void *stream);
@@ -318,7 +317,9 @@ int wmibm_force_mask(wmibm_handle *h, const void *const tau[6], void *fx, void *
  * mean "choose automatically".
  */
 typedef struct wmibm_tuning {
-    int32_t force_path;       /* 0 auto (as 3), 1 bulk-copy pipeline only, 2 direct-load kernel only,
+    int32_t force_path;       /* 0 auto (the direct-load kernel, or with rows, stages, consumer_warps,
+                                 blocks_per_sm or dyn_chunk set as 3), 1 bulk-copy pipeline only,
+                                 2 direct-load kernel only,
                                  3 bulk-copy pipeline with the wall model always in a kernel of its
                                  own (no single-launch step), 4 as 1 with the single-launch step's
                                  wall model in dedicated blocks (one per SM) instead of a share of
@@ -434,10 +435,10 @@ int wmibm_backward(wmibm_handle *h, const void *const g[3], const void *const uv
 /*
  * Batched ensembles: many terrains of uneven grid sizes stepped together.
  * The step of a batch is the per-step stage (wmibm_step without grad p) of
- * every member, done by two persistent launches over all members: the wall
- * kernel over the concatenated band records and solid runs, then the
- * pipelined force + body-mask kernel over the concatenated (member, strip,
- * level) units.  Member descriptors (field pointers) live in device memory, so
+ * every member, done by two launches over all members: the wall kernel over
+ * the concatenated band records and solid runs, then the force + body-mask
+ * kernel over the concatenated blocks of all members (or, tuned, the pipelined
+ * kernel over the (member, strip, level) units).  Member descriptors (field pointers) live in device memory, so
  * a step can be captured in a CUDA graph and replayed.
  */
 typedef struct wmibm_batch wmibm_batch;
@@ -464,8 +465,7 @@ int wmibm_batch_set_fields(wmibm_batch *b, const wmibm_member_fields *fields, vo
 
 /* Tile shape and form of the batch launches (force_path, rows, stages, consumer_warps,
  * wall_warps, blocks_per_sm, dyn_chunk, wall_grid used).  A batch that is never
- * tuned (every field 0) takes two launches, 4-row strips, two stages, four
- * consumer warps and runs of at least 16 units. */
+ * tuned (every field 0) takes the wall kernel and the direct-load stencil. */
 int wmibm_batch_set_tuning(wmibm_batch *b, const wmibm_tuning *t);
 
 /*

@@ -119,14 +119,27 @@ bool batch_config(wmibm_batch *b, StencilConfig *out, std::vector<int> *rows_out
     return true;
 }
 
-// Levels per chunk of the direct-load stencil's blocks.
-constexpr int kDirectBatchLevels = 2;
+// Levels per chunk of the direct-load stencil's blocks: long chunks pay a block's
+// look-up of its member less often, short ones leave enough blocks for the launch's
+// end.  The longest of 16, 4, 2 that leaves eight waves of blocks (step in us with
+// chunks of 2 / 4 / 16 levels: 64 members of 85 M nodes 607 / 593 / 575, 5 members
+// 42.1 / 42.1 / 45.5, 6 in FP64 323 / 326 / 340; the pipelined stencil: 597, 53.6
+// and 412).
+template <typename T>
+int direct_levels(const wmibm_batch *b)
+{
+    int64_t groups = 0;         // groups of the values a block holds, over all levels
+    for (const auto *h : b->members) groups += h->n / (256 * (16 / (int)sizeof(T)));
+    const int64_t waves = 8 * 3 * (int64_t)b->members[0]->sm_count;
+    return groups / 16 >= waves ? 16 : (groups / 4 >= waves ? 4 : 2);
+}
 
 template <typename T>
 int upload_members(wmibm_batch *b, const wmibm_member_fields *fields, cudaStream_t stream)
 {
     std::vector<Member<T>> host(b->count);
     int64_t c_off = 0, d_off = 0, r_off = 0, run_off = 0, body_off = 0, clean = 0, dirty = 0;
+    const int kc = direct_levels<T>(b);
     for (int m = 0; m < b->count; ++m) {
         wmibm_handle *h = b->members[m];
         const wmibm_member_fields &fl = fields[m];
@@ -138,7 +151,8 @@ int upload_members(wmibm_batch *b, const wmibm_member_fields *fields, cudaStream
         mm.r_off = r_off;
         mm.run_off = run_off;
         mm.body_off = body_off;
-        direct_tile(mm, 16 / (int)sizeof(T), 0, 0, kDirectBatchLevels);
+        direct_tile(mm, 16 / (int)sizeof(T), 0, 0, kc);
+        b->offsets.whole = (m == 0 || b->offsets.whole) && whole_sectors(mm);
         b->offsets.clean[m] = (int32_t)clean;
         b->offsets.dirty[m] = (int32_t)dirty;
         const int64_t tiles = (int64_t)mm.gx * mm.gy;

@@ -92,6 +92,7 @@ constexpr int kMaxBatchMembers = 256;
 // kernel parameter: the look-up runs on the constant bank).
 struct DirectBatch {
     int32_t clean[kMaxBatchMembers + 1], dirty[kMaxBatchMembers + 1];
+    int32_t whole;              // no 32-byte sector of any member's stresses holds values of two levels
 };
 
 template <typename T>
@@ -107,6 +108,9 @@ bool stencil_config(const wmibm_handle *h, const void *const tau[6], void *const
 // The direct-load stencil's tile of a member for vectors of v values: bx vectors by by rows, kc levels (0: chosen).
 template <typename T>
 void direct_tile(Member<T> &m, int v, int bx, int by, int kc);
+
+template <typename T>
+bool whole_sectors(const Member<T> &m);
 
 // The batch wall kernel, then the direct-load stencil over all members.
 template <typename T, typename VEL>

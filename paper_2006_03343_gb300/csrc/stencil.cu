@@ -1705,25 +1705,28 @@ template <typename T, int V>
 struct Vec {
     T v[V];
 };
-__device__ __forceinline__ Vec<float, 4> ldv(const float *p, Vec<float, 4> *)
+// NC: through the read-only path.
+template <bool NC, typename P>
+__device__ __forceinline__ P ld1(const P *p)
 {
-    const float4 a = *reinterpret_cast<const float4 *>(p);
-    return Vec<float, 4>{{a.x, a.y, a.z, a.w}};
+    if constexpr (NC) return __ldg(p);
+    else return *p;
 }
-__device__ __forceinline__ Vec<float, 2> ldv(const float *p, Vec<float, 2> *)
+template <bool NC, typename T, int V>
+__device__ __forceinline__ Vec<T, V> ldv(const T *p)
 {
-    const float2 a = *reinterpret_cast<const float2 *>(p);
-    return Vec<float, 2>{{a.x, a.y}};
-}
-__device__ __forceinline__ Vec<double, 2> ldv(const double *p, Vec<double, 2> *)
-{
-    const double2 a = *reinterpret_cast<const double2 *>(p);
-    return Vec<double, 2>{{a.x, a.y}};
-}
-template <typename T>
-__device__ __forceinline__ Vec<T, 1> ldv(const T *p, Vec<T, 1> *)
-{
-    return Vec<T, 1>{{*p}};
+    if constexpr (V * sizeof(T) == 16 && sizeof(T) == 4) {
+        const float4 a = ld1<NC>(reinterpret_cast<const float4 *>(p));
+        return Vec<T, V>{{a.x, a.y, a.z, a.w}};
+    } else if constexpr (V == 2 && sizeof(T) == 4) {
+        const float2 a = ld1<NC>(reinterpret_cast<const float2 *>(p));
+        return Vec<T, V>{{a.x, a.y}};
+    } else if constexpr (V == 2) {
+        const double2 a = ld1<NC>(reinterpret_cast<const double2 *>(p));
+        return Vec<T, V>{{a.x, a.y}};
+    } else {
+        return Vec<T, V>{{ld1<NC>(p)}};
+    }
 }
 __device__ __forceinline__ void stv(float *p, const Vec<float, 4> &x)
 {
@@ -1758,6 +1761,8 @@ constexpr int kDirectBlocks = sizeof(T) == 4 && V <= 2 ? 4 : 3;
 
 struct NoBatch {
 };
+// The forcing alone; after a wall launch; the same with dirty levels' stresses in a buffer of their own.
+constexpr int kDirectPlain = 0, kDirectAfter = 1, kDirectSplit = 2;
 
 // f = -div(tau) with loads through L1 (periodic central differences, Eqs. 15-16 in
 // z), the stencil of untuned launches.  A thread owns V consecutive x-points of one
@@ -1777,14 +1782,16 @@ struct NoBatch {
 // After a wall launch (AFTER) the grid is a programmatic dependent of it: blocks of
 // clean chunks come first and start at once, those of dirty chunks wait for the wall
 // kernel, and the tail's blocks apply the body mask (Eq. 27) and convert the
-// statistics after the same wait.  BATCH: the blocks of all members, clean ones
-// first.  Loads are not of the read-only kind: an SM's cache may hold what a clean
-// block read of a sector that a dirty level's first row shares.
-template <typename T, typename VEL, int V, bool AFTER, typename Batch>
+// statistics after the same wait.  Batch: the blocks of all members, clean ones
+// first.  NC: loads through the read-only path (hill step 207 -> 183 us: the compiler
+// keeps more of them in flight).  Not where a 32-byte sector holds values of two
+// levels: an SM's cache may then keep what a clean block read of it from before the
+// wall kernel wrote the dirty level's part.
+template <typename T, typename VEL, int V, int KIND, bool NC, typename Batch>
 __global__ void __launch_bounds__(kDirectThreads, (kDirectBlocks<T, V>))
     k_direct(const __grid_constant__ KParams<T> p, const __grid_constant__ Batch batch)
 {
-    constexpr bool BATCH = !std::is_same<Batch, NoBatch>::value;
+    constexpr bool BATCH = !std::is_same<Batch, NoBatch>::value, AFTER = KIND != kDirectPlain;
     using W = Vec<T, V>;
     int b = blockIdx.x;
     const int t = threadIdx.x;
@@ -1799,7 +1806,20 @@ __global__ void __launch_bounds__(kDirectThreads, (kDirectBlocks<T, V>))
     }
     const bool dirty = AFTER && b >= p.clean_blocks;
     if (dirty) b -= p.clean_blocks;
-    const Member<T> *mm = &p.one;
+    // the member's arrays and shape: kernel parameters, or (BATCH) registers
+    const T *q[6];
+    T *fq[3];
+    int nx, ny, nz, bx, by, gx, gy, kc, dc0, dcn;
+    T cx, cy, cz;
+    auto take = [&](const Member<T> &m) {
+#pragma unroll
+        for (int a = 0; a < 6; ++a) q[a] = m.tau[a];
+#pragma unroll
+        for (int a = 0; a < 3; ++a) fq[a] = m.f[a];
+        nx = m.nx; ny = m.ny; nz = m.nz;
+        bx = m.bx; by = m.by; gx = m.gx; gy = m.gy; kc = m.kc; dc0 = m.dc0; dcn = m.dcn;
+        cx = m.cx; cy = m.cy; cz = m.cz;
+    };
     if constexpr (BATCH) {
         const int32_t *first = dirty ? batch.dirty : batch.clean;
         int lo = 0, hi = p.nmembers - 1;
@@ -1809,59 +1829,59 @@ __global__ void __launch_bounds__(kDirectThreads, (kDirectBlocks<T, V>))
             else hi = mid - 1;
         }
         b -= first[lo];
-        mm = p.list + lo;
+        take(p.list[lo]);
+    } else {
+        take(p.one);
     }
-    const Member<T> &m = *mm;
-    const int nx = m.nx, ny = m.ny, nz = m.nz, bx = m.bx, gx = m.gx, kc = m.kc;
-    const int tiles = gx * m.gy;
+    const int tiles = gx * gy;
     int c = b / tiles;
     const int tile = b - c * tiles, tile_y = tile / gx, tile_x = tile - tile_y * gx;
-    if (dirty) c += m.dc0;
-    else if (c >= m.dc0) c += m.dcn;
-    const int ly = t / bx, by = m.by;
+    if (dirty) c += dc0;
+    else if (c >= dc0) c += dcn;
+    const int ly = t / bx;
     const int i = (tile_x * bx + (t - ly * bx)) * V, j = tile_y * by + ly;
     // what follows this launch in the stream relies on the wall kernel's end as well
-    if (AFTER && (dirty || blockIdx.x == gridDim.x - 1)) {
-        wait_wall_kernel();
-        __threadfence();
-    }
+    if (AFTER && (dirty || blockIdx.x == gridDim.x - 1)) wait_wall_kernel();
     if (ly >= by || i >= nx || j >= ny) return;
     const int k0 = c * kc, k1 = min(k0 + kc, nz), plane = nx * ny;
     const int im = (i == 0) ? nx - 1 : i - 1, ip = (i + V == nx) ? 0 : i + V;
     const int jm = (j == 0) ? ny - 1 : j - 1, jp = (j + 1 == ny) ? 0 : j + 1;
     const int at = j * nx + i, atm = jm * nx + i, atp = jp * nx + i, left = j * nx + im, right = j * nx + ip;
-    const T cx = m.cx, cy = m.cy, cz = m.cz;
-    T *const fx = m.f[0], *const fy = m.f[1], *const fz = m.f[2];
-    auto field = [&](int a, bool own) -> const T * { return (BATCH || own) ? m.tau[a] : m.tin[a]; };
-    const bool own0 = k0 >= m.da && k0 < m.db;
-    W xz_k = ldv(field(4, own0) + k0 * plane + at, (W *)nullptr);
-    W yz_k = ldv(field(5, own0) + k0 * plane + at, (W *)nullptr);
+    // SPLIT: which of the two sets of stresses a level is read from
+    auto choose = [&](int k) {
+        if (KIND != kDirectSplit) return;
+        const bool own = k >= p.one.da && k < p.one.db;
+#pragma unroll
+        for (int a = 0; a < 6; ++a) q[a] = own ? p.one.tau[a] : p.one.tin[a];
+    };
+    choose(k0);
+    W xz_k = ldv<NC, T, V>(q[4] + k0 * plane + at);
+    W yz_k = ldv<NC, T, V>(q[5] + k0 * plane + at);
     W zz_km;
     for (int e = 0; e < V; ++e) zz_km.v[e] = T(0);
-    if (k0 > 0) zz_km = ldv(field(3, own0) + (k0 - 1) * plane + at, (W *)nullptr);
+    if (k0 > 0) zz_km = ldv<NC, T, V>(q[3] + (k0 - 1) * plane + at);
     for (int k = k0; k < k1; ++k) {
-        const bool own = k >= m.da && k < m.db, top = k == nz - 1;
+        choose(k);
+        const bool top = k == nz - 1;
         const int o = k * plane, up = top ? o : o + plane;
-        const T *const txx = field(0, own) + o, *const txy = field(1, own) + o, *const tyy = field(2, own) + o;
-        const T *const tzz = field(3, own) + o, *const txz = field(4, own), *const tyz = field(5, own);
         Level<T, V> l;
-        l.xx = ldv(txx + at, (W *)nullptr);
-        l.xxl = txx[left];
-        l.xxr = txx[right];
-        l.xy = ldv(txy + at, (W *)nullptr);
-        l.xyl = txy[left];
-        l.xyr = txy[right];
-        l.xyjm = ldv(txy + atm, (W *)nullptr);
-        l.xyjp = ldv(txy + atp, (W *)nullptr);
-        l.yyjm = ldv(tyy + atm, (W *)nullptr);
-        l.yyjp = ldv(tyy + atp, (W *)nullptr);
-        l.yzjm = ldv(tyz + o + atm, (W *)nullptr);
-        l.yzjp = ldv(tyz + o + atp, (W *)nullptr);
-        l.xzl = txz[o + left];
-        l.xzr = txz[o + right];
-        l.zz = ldv(tzz + at, (W *)nullptr);
-        l.xz_kp = ldv(txz + up + at, (W *)nullptr);
-        l.yz_kp = ldv(tyz + up + at, (W *)nullptr);
+        l.xx = ldv<NC, T, V>(q[0] + o + at);
+        l.xxl = ld1<NC>(q[0] + o + left);
+        l.xxr = ld1<NC>(q[0] + o + right);
+        l.xy = ldv<NC, T, V>(q[1] + o + at);
+        l.xyl = ld1<NC>(q[1] + o + left);
+        l.xyr = ld1<NC>(q[1] + o + right);
+        l.xyjm = ldv<NC, T, V>(q[1] + o + atm);
+        l.xyjp = ldv<NC, T, V>(q[1] + o + atp);
+        l.yyjm = ldv<NC, T, V>(q[2] + o + atm);
+        l.yyjp = ldv<NC, T, V>(q[2] + o + atp);
+        l.yzjm = ldv<NC, T, V>(q[5] + o + atm);
+        l.yzjp = ldv<NC, T, V>(q[5] + o + atp);
+        l.xzl = ld1<NC>(q[4] + o + left);
+        l.xzr = ld1<NC>(q[4] + o + right);
+        l.zz = ldv<NC, T, V>(q[3] + o + at);
+        l.xz_kp = ldv<NC, T, V>(q[4] + up + at);
+        l.yz_kp = ldv<NC, T, V>(q[5] + up + at);
         W Fx, Fy, Fz;
 #pragma unroll
         for (int e = 0; e < V; ++e) {
@@ -1875,9 +1895,9 @@ __global__ void __launch_bounds__(kDirectThreads, (kDirectBlocks<T, V>))
             Fy.v[e] = top ? T(0) : vy;
             Fz.v[e] = (top || k == 0) ? T(0) : vz;
         }
-        stv(fx + o + at, Fx);
-        stv(fy + o + at, Fy);
-        stv(fz + o + at, Fz);
+        stv(fq[0] + o + at, Fx);
+        stv(fq[1] + o + at, Fy);
+        stv(fq[2] + o + at, Fz);
         xz_k = l.xz_kp;
         yz_k = l.yz_kp;
         zz_km = l.zz;
@@ -2085,13 +2105,13 @@ int launch_wall_single(wmibm_handle *h, void *const tau[6], const void *u, const
 
 // The direct-load stencil over p's member(s): its grid, then the launch.  body_total,
 // do_mask and emit_stats are the tail's work; pdl: the wall kernel comes just before.
-template <typename T, typename VEL, int V, bool AFTER, typename Batch>
+template <typename T, typename VEL, int V, int KIND, bool NC, typename Batch>
 int launch_direct(wmibm_handle *h, KParams<T> &p, const Batch &batch, bool pdl, cudaStream_t stream)
 {
     const int64_t want = (p.body_total + 2 * kDirectThreads - 1) / (2 * kDirectThreads);
     p.tail_blocks = p.do_mask ? (int32_t)std::min<int64_t>(want, 4 * (int64_t)h->sm_count) : 0;
     if (p.emit_stats && p.tail_blocks == 0) p.tail_blocks = 1;
-    if (!AFTER) p.tail_blocks = 0;
+    if (KIND == kDirectPlain) p.tail_blocks = 0;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3((unsigned)(p.clean_blocks + p.dirty_blocks + p.tail_blocks));
     cfg.blockDim = dim3(kDirectThreads);
@@ -2100,8 +2120,8 @@ int launch_direct(wmibm_handle *h, KParams<T> &p, const Batch &batch, bool pdl, 
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
-    cfg.numAttrs = AFTER && pdl ? 1 : 0;
-    return cuda_status(h, cudaLaunchKernelEx(&cfg, k_direct<T, VEL, V, AFTER, Batch>, p, batch), "k_direct launch");
+    cfg.numAttrs = KIND != kDirectPlain && pdl ? 1 : 0;
+    return cuda_status(h, cudaLaunchKernelEx(&cfg, k_direct<T, VEL, V, KIND, NC, Batch>, p, batch), "k_direct launch");
 }
 
 // Values per vector that every row of these arrays is aligned for.
@@ -2118,7 +2138,7 @@ int direct_vector(const Member<T> &m)
     return 1;
 }
 
-template <typename T, typename VEL, bool AFTER>
+template <typename T, typename VEL, int KIND>
 int direct_single(wmibm_handle *h, KParams<T> &p, bool pdl, cudaStream_t stream)
 {
     const int v = direct_vector(p.one);
@@ -2127,11 +2147,16 @@ int direct_single(wmibm_handle *h, KParams<T> &p, bool pdl, cudaStream_t stream)
     if (tiles * chunks > INT32_MAX / 2) return set_error(h, WMIBM_EINVAL, "grid too large for the force launch");
     p.clean_blocks = (int32_t)(tiles * (chunks - p.one.dcn));
     p.dirty_blocks = (int32_t)(tiles * p.one.dcn);
-    if constexpr (sizeof(T) == 4) {
-        if (v == 4) return launch_direct<T, VEL, 4, AFTER>(h, p, NoBatch{}, pdl, stream);
+    constexpr int kWide = 16 / (int)sizeof(T);
+    if (v == kWide) {
+        if (KIND == kDirectPlain || whole_sectors(p.one))
+            return launch_direct<T, VEL, kWide, KIND, true>(h, p, NoBatch{}, pdl, stream);
+        return launch_direct<T, VEL, kWide, KIND, false>(h, p, NoBatch{}, pdl, stream);
     }
-    if (v == 2) return launch_direct<T, VEL, 2, AFTER>(h, p, NoBatch{}, pdl, stream);
-    return launch_direct<T, VEL, 1, AFTER>(h, p, NoBatch{}, pdl, stream);
+    if constexpr (sizeof(T) == 4) {
+        if (v == 2) return launch_direct<T, VEL, 2, KIND, false>(h, p, NoBatch{}, pdl, stream);
+    }
+    return launch_direct<T, VEL, 1, KIND, false>(h, p, NoBatch{}, pdl, stream);
 }
 
 template <typename T, typename VEL>
@@ -2146,13 +2171,26 @@ int direct_impl(wmibm_handle *h, const void *const tau[6], const void *const own
     p.do_mask = do_mask;
     p.stats = emit;
     p.emit_stats = emit != nullptr;
-    if (after) return direct_single<T, VEL, true>(h, p, pdl, stream);
-    return direct_single<T, T, false>(h, p, false, stream);      // no mask: the velocity's type does not matter
+    // without a mask the velocity's type does not matter
+    if (!after) return direct_single<T, T, kDirectPlain>(h, p, false, stream);
+    if (own != tau) return direct_single<T, T, kDirectSplit>(h, p, pdl, stream);
+    return direct_single<T, VEL, kDirectAfter>(h, p, pdl, stream);
 }
 
 }  // namespace
 
 namespace wmibm {
+
+// Whether no 32-byte sector holds values of two levels.
+template <typename T>
+bool whole_sectors(const Member<T> &m)
+{
+    bool whole = (int64_t)m.nx * m.ny * (int64_t)sizeof(T) % 32 == 0;
+    for (int a = 0; a < 6; ++a) whole = whole && ((uintptr_t)m.tau[a] & 31u) == 0 && ((uintptr_t)m.tin[a] & 31u) == 0;
+    return whole;
+}
+template bool whole_sectors<float>(const Member<float> &);
+template bool whole_sectors<double>(const Member<double> &);
 
 template <typename T>
 void direct_tile(Member<T> &m, int v, int bx, int by, int kc)
@@ -2509,8 +2547,11 @@ int batch_launch_direct(wmibm_handle *h0, const Member<T> *dev_members, int nmem
     int st = launch_wall_batch<T, VEL>(h0, p, c, 0, stream);
     if (st) return st;
     constexpr int V = 16 / (int)sizeof(T);
-    if (nmembers == 1) return launch_direct<T, VEL, V, true>(h0, p, NoBatch{}, true, stream);
-    return launch_direct<T, VEL, V, true>(h0, p, offsets, true, stream);
+    if (nmembers == 1)
+        return offsets.whole ? launch_direct<T, VEL, V, kDirectAfter, true>(h0, p, NoBatch{}, true, stream)
+                             : launch_direct<T, VEL, V, kDirectAfter, false>(h0, p, NoBatch{}, true, stream);
+    return offsets.whole ? launch_direct<T, VEL, V, kDirectAfter, true>(h0, p, offsets, true, stream)
+                         : launch_direct<T, VEL, V, kDirectAfter, false>(h0, p, offsets, true, stream);
 }
 
 template int batch_launch_direct<float, float>(wmibm_handle *, const Member<float> *, int, const KParams<float> &,
