@@ -404,8 +404,8 @@ int wmibm_wall_stress_noalloc(wmibm_handle *h, const void *u, const void *v, con
  * Every later wmibm_wall_stress, wmibm_wall_stress_noalloc, wmibm_step,
  * wmibm_wall_stress_force and batch step of this handle computes C per node
  * from it.  The first call also builds the transpose of the band records'
- * trilinear gathers (host sort of 16 entries per band node, then upload; it
- * synchronizes `stream`), so make it before any stream capture.
+ * trilinear gathers (16 entries per band node; it allocates and synchronizes
+ * `stream`), so make it before any stream capture.
  * Errors: EINVAL (misaligned logz0, more than 2^27 band nodes), ESTATE,
  * ENOMEM, ECUDA.
  */
