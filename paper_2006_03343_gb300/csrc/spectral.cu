@@ -16,10 +16,12 @@
 //               terms -> writes the partial forcing into f
 //   column unit (level k, wy columns): d_y of txy, tyy, tyz, subtracted from f
 // Each unit stages its lines in shared memory, two real lines per complex
-// sequence (z = a + i b; the derivative operator is real, so D z = D a + i D b),
-// runs a radix-16/8/4/2 Stockham FFT, multiplies by i k / N while loading the first
-// pass of a second forward FFT of the conjugate (IFFT(y) = conj(FFT(conj y))/N),
-// and writes.  Units are dispensed by an atomic ticket in chunks of kc levels:
+// sequence (z = a + i b; the derivative operator is real, so D z = D a + i D b), runs
+// a decimation-in-frequency FFT in place (radix up to 16), whose last pass leaves the
+// bins in digit-reversed order, multiplies them there by i k / N and conjugates them
+// (IFFT(y) = conj(FFT(conj y))/N), and runs the transposed network, whose first pass
+// takes the same elements: the two passes are one, no reordering is needed, and the
+// result is in natural order.  Units are dispensed by an atomic ticket in chunks of kc levels:
 // the row units of chunk c, then the column units of chunk c-1.  A column unit
 // on level k waits (bounded) until all row units of level k have finished, so
 // the partial forcing and the stresses the two unit kinds share are re-read
@@ -35,8 +37,8 @@
 namespace wmibm {
 
 constexpr int kSpecMaxLog = 11;         // lines of up to 2048 points (FP32; 1024 for FP64)
-constexpr int kSpecThreads = 256;
-constexpr int kSpecBudget = 3200;       // complex elements per shared buffer aimed at (FP32; half for FP64)
+constexpr int kSpecThreads = 192;
+constexpr int kSpecBudget = 3300;       // complex elements per shared buffer aimed at (FP32; half for FP64)
 constexpr double kSpecChunkBytes = 24.0 * 1024 * 1024;   // L2 footprint of one chunk of levels
 
 struct SpecState {
@@ -46,9 +48,10 @@ struct SpecState {
     int kc, nchunks;
     int xpl, ypl;               // units per level
     int64_t total;
+    int64_t buf;                // complex elements of the FFT buffer
     size_t smem;
-    void *twx, *twy;            // omega_N^m = exp(-2 pi i m / N), m < N (dtype complex)
-    void *knx, *kny;            // k_m / N per bin, Nyquist bin 0 (dtype)
+    void *twx, *twy;            // twiddles of the passes (dtype complex)
+    void *knx, *kny;            // k_m / N per bin in the FFT's digit-reversed order, Nyquist bin 0 (dtype)
     unsigned int *ctr;          // [0] ticket, [1] exit ticket, [2 + k] row units finished on level k
 };
 
@@ -82,7 +85,7 @@ struct SpecParams {
     int32_t ldx, ldy;
     int32_t kc, nchunks, xpl, ypl;
     int64_t total;
-    int32_t buf;              // complex elements per shared buffer
+    int32_t buf;              // complex elements of the FFT buffer
     int32_t v16;              // stage with 16-byte copies (every staged segment 16-byte aligned)
     T rdz;
 };
@@ -96,23 +99,23 @@ __device__ __forceinline__ C cmul(C a, C b) { return C{a.x * b.x - a.y * b.y, a.
 template <typename C>
 __device__ __forceinline__ C cmi(C a) { return C{a.y, -a.x}; }       // -i a
 
-// Element e of a sequence sits at e + e/32 in shared memory: the padding spreads
-// the stride-R writes of the first Stockham pass over the banks.
-__device__ __forceinline__ int sk(int e) { return e + (e >> 5); }
+// Element e of a sequence sits at e + e/16 in shared memory: passes of stride 16 and
+// more read 16 consecutive elements to a half-warp, and the middle pass, whose
+// butterflies take R consecutive elements each, a different bank for each of them.
+__device__ __forceinline__ int sk(int e) { return e + (e >> 4); }
 
-// log2 of the radix of the Stockham pass that starts at Ns = 2^logns in a
-// transform of N = 2^logn points: as few passes as radix 2^maxlog allows, the
-// first at the largest radix and the others as even as possible (FP32, radix up
-// to 16: 256 = 16 x 16, 512 = 16 x 8 x 4, 1024 = 16 x 8 x 8; FP64, whose values
-// take twice the registers: radix up to 8).  A first pass of radix 16 keeps the
-// second pass's stride at Ns = 16: with the one-per-32 skew its stores spread
-// two lanes to an 8-byte bank slot, where Ns = 8 (512 = 8 x 8 x 8) put four.
-__host__ __device__ constexpr int pass_log(int logn, int logns, int maxlog)
+// The passes of an N = 2^logn point transform: outer ones of radix 2^outer_log, each on
+// the blocks that the ones before it left, then the middle one of radix 2^mid_log on
+// consecutive elements, as large as maxlog allows (it does two DFTs on one trip through
+// shared memory); as few outer ones as maxlog allows, as even as possible, and at least
+// one (FP32, radix up to 16: 256 = 16 x 16, 512 = 8 x 4 x 16; FP64, whose values take
+// twice the registers: up to 8).
+__host__ __device__ constexpr int mid_log(int logn, int maxlog) { return logn <= maxlog ? logn - 1 : maxlog; }
+__host__ __device__ constexpr int outer_log(int logn, int used, int maxlog)
 {
-    return logn - logns <= 0 ? 0
-           : logns == 0      ? (logn < maxlog ? logn : maxlog)
-                             : (logn - logns + (logn - logns + maxlog - 1) / maxlog - 1) /
-                                   ((logn - logns + maxlog - 1) / maxlog);
+    const int left = logn - mid_log(logn, maxlog) - used;
+    const int passes = (left + maxlog - 1) / maxlog;
+    return left <= 0 ? 0 : (left + passes - 1) / passes;
 }
 template <typename T>
 constexpr int kMaxPassLog = sizeof(T) == 4 ? 4 : 3;
@@ -121,6 +124,14 @@ constexpr int kMaxPassLog = sizeof(T) == 4 ? 4 : 3;
 // V[q] = sum_r v[r] exp(-2 pi i r q / R).
 template <typename T, int R>
 struct Dft;
+
+template <typename T>
+struct Dft<T, 1> {
+    template <typename C>
+    __device__ __forceinline__ static void run(C *)
+    {
+    }
+};
 
 template <typename T>
 struct Dft<T, 2> {
@@ -206,115 +217,113 @@ struct Dft<T, 8> {
     }
 };
 
-// The R outputs of a first-pass butterfly (Ns = 1: element r of the butterfly at
-// out[r]).  With R = 16 the elements of butterfly j start at 16 j + j/2 under the
-// skew, so butterflies j and j + 1 of a half-warp share their 8-byte bank slots:
-// an odd j writes its upper half first, which spreads each store's 16 lanes over
-// 16 slots (FP32, NB >= 16: a half-warp holds 16 butterflies of one sequence).
-template <typename T, int R, int NB, typename C>
-__device__ __forceinline__ void store_first_pass(C *out, const C *v, int j)
-{
-    constexpr bool kRot = sizeof(T) == 4 && R == 16 && NB >= 16;
-    if (kRot) {
-        const bool odd = (j & 1) != 0;
-        C *const lo = out + (odd ? R / 2 : 0), *const hi = out - (odd ? R / 2 : 0);
-#pragma unroll
-        for (int i = 0; i < R / 2; ++i) lo[i] = odd ? v[i + R / 2] : v[i];
-#pragma unroll
-        for (int i = R / 2; i < R; ++i) hi[i] = odd ? v[i - R / 2] : v[i];
-    } else {
-#pragma unroll
-        for (int r = 0; r < R; ++r) out[r] = v[r];
-    }
-}
-
-// One Stockham pass of radix R = 2^pass_log(LOGN, LOGNS, kMaxPassLog<T>) over S sequences of length
-// N = 2^LOGN, from a to b, after passes that reached Ns = 2^LOGNS.  Butterfly j
-// of a sequence reads elements j + r N/R, twiddles them by
-// omega_N^(r jm N/(Ns R)) with jm = j mod Ns, and writes element
-// (j - jm) R + jm + r Ns.  The pass's twiddles are a table of its own,
-// tw[(r - 1) Ns + jm], so that a warp's loads of one r are contiguous.  With N
-// and Ns known at compile time every shared address is a base plus an
-// immediate: since N/R and Ns divide 32 or are multiples of it,
-// sk(j + r N/R) = sk(j) + r N/R + (r N/R)/32 and sk(o0 + r Ns) = sk(o0) + r Ns + (r Ns)/32.
-// PRE: multiply each input (bin m) by i k_m / N and conjugate it first, i.e.
-// v -> (-kn_m v.y, -kn_m v.x).
-template <typename T, int LOGN, int LOGNS, bool PRE>
-__device__ __forceinline__ void fft_pass(const typename Cx<T>::type *__restrict__ a,
-                                         typename Cx<T>::type *__restrict__ b, int S, int ld,
-                                         const typename Cx<T>::type *__restrict__ tw, const T *__restrict__ kn)
+// One outer pass, in place, after passes of radices that multiply to 2^USED: on every
+// block of M = N / 2^USED elements, butterfly j < M / R takes the elements j + r M / R.
+// FORWARD: DFT, then the twiddles omega_M^(j q) on its outputs; the transposed pass:
+// the same twiddles on its inputs, then the DFT.  The pass's twiddles are a table of
+// its own, tw[(q - 1) M / R + j], so that a warp's loads of one q are contiguous.
+// Every shared address is a base plus an immediate: M / R divides 16 or is a multiple
+// of it, so sk(e + r M / R) = sk(e) + r M / R + (r M / R) / 16.
+template <typename T, int LOGN, int USED, bool FORWARD>
+__device__ __forceinline__ void outer_pass(typename Cx<T>::type *a, int S, int ld,
+                                           const typename Cx<T>::type *__restrict__ tw)
 {
     using C = typename Cx<T>::type;
-    constexpr int LOGR = pass_log(LOGN, LOGNS, kMaxPassLog<T>);
-    constexpr int R = 1 << LOGR;
-    constexpr int LOGNB = LOGN - LOGR;
-    constexpr int NB = 1 << LOGNB;
-    constexpr int NS = 1 << LOGNS;
+    constexpr int LOGR = outer_log(LOGN, USED, kMaxPassLog<T>), R = 1 << LOGR;
+    constexpr int LOGNB = LOGN - LOGR, LOGSTEP = LOGN - USED - LOGR, STEP = 1 << LOGSTEP;
     const int total = S << LOGNB;
     for (int t = threadIdx.x; t < total; t += kSpecThreads) {
-        const int s = t >> LOGNB, j = t & (NB - 1);
-        const C *in = a + s * ld + sk(j);
+        const int s = t >> LOGNB, jj = t & ((1 << LOGNB) - 1);
+        const int j = jj & (STEP - 1), block = jj >> LOGSTEP;
+        C *const at = a + s * ld + sk((block << (LOGN - USED)) + j);
+        const C *const w = tw + j;
         C v[R];
 #pragma unroll
-        for (int r = 0; r < R; ++r) v[r] = in[r * NB + ((r * NB) >> 5)];
-        if (PRE) {
-            const T *k0 = kn + j;
+        for (int r = 0; r < R; ++r) v[r] = at[r * STEP + ((r * STEP) >> 4)];
+        if (!FORWARD) {
 #pragma unroll
-            for (int r = 0; r < R; ++r) {
-                const T k = __ldg(k0 + r * NB);
-                v[r] = C{-k * v[r].y, -k * v[r].x};
-            }
-        }
-        const int jm = j & (NS - 1);
-        if (LOGNS > 0) {
-            const typename Cx<T>::type *w0 = tw + jm;
-#pragma unroll
-            for (int r = 1; r < R; ++r) v[r] = cmul(v[r], __ldg(w0 + (r - 1) * NS));
+            for (int q = 1; q < R; ++q) v[q] = cmul(v[q], __ldg(w + (q - 1) * STEP));
         }
         Dft<T, R>::run(v);
-        C *out = b + s * ld + sk(((j - jm) << LOGR) + jm);
-        if (LOGNS == 0) {
-            store_first_pass<T, R, NB>(out, v, j);
-        } else {
+        if (FORWARD) {
 #pragma unroll
-            for (int r = 0; r < R; ++r) out[r * NS + ((r * NS) >> 5)] = v[r];
+            for (int q = 1; q < R; ++q) v[q] = cmul(v[q], __ldg(w + (q - 1) * STEP));
         }
+#pragma unroll
+        for (int r = 0; r < R; ++r) at[r * STEP + ((r * STEP) >> 4)] = v[r];
     }
 }
 
-// The remaining passes of a transform, from Ns = 2^LOGNS on, ping-ponging
-// between a and b with a block barrier after each; returns the buffer that holds
-// the result.  tw points at the table of the pass that starts at LOGNS.
-template <typename T, int LOGN, int LOGNS, bool PRE>
-struct Passes {
-    using C = typename Cx<T>::type;
-    __device__ __forceinline__ static C *run(C *a, C *b, int S, int ld, const C *tw, const T *kn)
-    {
-        constexpr int LOGR = pass_log(LOGN, LOGNS, kMaxPassLog<T>);
-        fft_pass<T, LOGN, LOGNS, PRE>(a, b, S, ld, tw, kn);
-        __syncthreads();
-        return Passes<T, LOGN, LOGNS + LOGR, false>::run(b, a, S, ld, tw + (((1 << LOGR) - 1) << LOGNS), kn);
-    }
-};
-template <typename T, int LOGN, bool PRE>
-struct Passes<T, LOGN, LOGN, PRE> {
-    using C = typename Cx<T>::type;
-    __device__ __forceinline__ static C *run(C *a, C *, int, int, const C *, const T *) { return a; }
-};
-
-// The first Stockham pass (Ns = 1, no twiddles) of the first transform, read
-// straight from the planar staging P (planes of n = L x N values): sequence s < L
-// is plane0 + i plane1 of line s, sequence L + q is plane 2 of lines 2q and 2q + 1.
-// ROWS: the staging is [line][pos] and consecutive threads take consecutive
-// butterflies of one sequence; otherwise it is [pos][line] and consecutive
-// threads take consecutive sequences of one butterfly, so that both the staging
-// reads and the skewed sequence writes stay spread over the banks.
-template <typename T, int LOGN, bool ROWS>
-__device__ __forceinline__ void fft_first_pass(const T *__restrict__ P, typename Cx<T>::type *__restrict__ b,
-                                               int logL, int ld)
+// The middle pass, in place: on R consecutive elements the forward transform's last
+// DFT, the bins' i k / N and conjugation, v -> (-kn v.y, -kn v.x), and the first DFT
+// of the second transform.  kn: in the order of the elements.
+template <typename T, int LOGN>
+__device__ __forceinline__ void mid_pass(typename Cx<T>::type *a, int S, int ld, const T *__restrict__ kn)
 {
     using C = typename Cx<T>::type;
-    constexpr int LOGR = pass_log(LOGN, 0, kMaxPassLog<T>);
+    constexpr int LOGR = mid_log(LOGN, kMaxPassLog<T>), R = 1 << LOGR, LOGNB = LOGN - LOGR;
+    const int total = S << LOGNB;
+    for (int t = threadIdx.x; t < total; t += kSpecThreads) {
+        const int s = t >> LOGNB, e = (t & ((1 << LOGNB) - 1)) << LOGR;
+        C *const at = a + s * ld + sk(e);
+        const T *const k = kn + e;
+        C v[R];
+#pragma unroll
+        for (int r = 0; r < R; ++r) v[r] = at[r];
+        Dft<T, R>::run(v);
+#pragma unroll
+        for (int r = 0; r < R; ++r) {
+            const T kr = __ldg(k + r);
+            v[r] = C{-kr * v[r].y, -kr * v[r].x};
+        }
+        Dft<T, R>::run(v);
+#pragma unroll
+        for (int r = 0; r < R; ++r) at[r] = v[r];
+    }
+}
+
+// The passes from the one after 2^USED on to the same one of the transposed network,
+// with a block barrier after each.  tw points at the table of the pass after 2^USED.
+template <typename T, int LOGN, int USED, bool MID>
+struct Passes {
+    using C = typename Cx<T>::type;
+    __device__ __forceinline__ static void run(C *a, int S, int ld, const C *tw, const T *kn)
+    {
+        constexpr int LOGR = outer_log(LOGN, USED, kMaxPassLog<T>), NEXT = USED + LOGR;
+        outer_pass<T, LOGN, USED, true>(a, S, ld, tw);
+        __syncthreads();
+        inner(a, S, ld, tw + (((1 << LOGR) - 1) << (LOGN - NEXT)), kn);
+        outer_pass<T, LOGN, USED, false>(a, S, ld, tw);
+        __syncthreads();
+    }
+    __device__ __forceinline__ static void inner(C *a, int S, int ld, const C *tw, const T *kn)
+    {
+        constexpr int NEXT = USED + outer_log(LOGN, USED, kMaxPassLog<T>);
+        Passes<T, LOGN, NEXT, (NEXT + mid_log(LOGN, kMaxPassLog<T>) == LOGN)>::run(a, S, ld, tw, kn);
+    }
+};
+template <typename T, int LOGN, int USED>
+struct Passes<T, LOGN, USED, true> {
+    using C = typename Cx<T>::type;
+    __device__ __forceinline__ static void run(C *a, int S, int ld, const C *, const T *kn)
+    {
+        mid_pass<T, LOGN>(a, S, ld, kn);
+        __syncthreads();
+    }
+};
+
+// The first outer pass, read straight from the planar staging P (planes of n = L x N
+// values): sequence s < L is plane0 + i plane1 of line s, sequence L + q is plane 2 of
+// lines 2q and 2q + 1.  ROWS: the staging is [line][pos] and consecutive threads take
+// consecutive butterflies of one sequence; otherwise it is [pos][line] and consecutive
+// threads take consecutive sequences of one butterfly, so that both the staging reads
+// and the skewed sequence writes stay spread over the banks.
+template <typename T, int LOGN, bool ROWS>
+__device__ __forceinline__ void first_pass(const T *__restrict__ P, typename Cx<T>::type *__restrict__ b, int logL,
+                                           int ld, const typename Cx<T>::type *__restrict__ tw)
+{
+    using C = typename Cx<T>::type;
+    constexpr int LOGR = outer_log(LOGN, 0, kMaxPassLog<T>);
     constexpr int R = 1 << LOGR;
     constexpr int LOGNB = LOGN - LOGR;
     constexpr int NB = 1 << LOGNB;
@@ -327,9 +336,13 @@ __device__ __forceinline__ void fft_first_pass(const T *__restrict__ P, typename
         if (ROWS) {
             s = t >> LOGNB;
             j = t & (NB - 1);
+        } else if (t < L << LOGNB) {            // the line sequences, then the plane-2 ones
+            j = t >> logL;
+            s = t & (L - 1);
         } else {
-            j = t / S;
-            s = t - j * S;
+            const int u = t - (L << LOGNB);
+            j = u >> (logL - 1);
+            s = L + (u & (L / 2 - 1));
         }
         C v[R];
         if (s < L) {
@@ -351,50 +364,49 @@ __device__ __forceinline__ void fft_first_pass(const T *__restrict__ P, typename
             }
         }
         Dft<T, R>::run(v);
-        C *out = b + s * ld + sk(j * R);
-        if (ROWS) {
-            store_first_pass<T, R, NB>(out, v, j);
-        } else {
+        const C *const w = tw + j;
 #pragma unroll
-            for (int r = 0; r < R; ++r) out[r] = v[r];
-        }
+        for (int q = 1; q < R; ++q) v[q] = cmul(v[q], __ldg(w + (q - 1) * NB));
+        C *const out = b + s * ld + sk(j);
+#pragma unroll
+        for (int q = 0; q < R; ++q) out[q * NB + ((q * NB) >> 4)] = v[q];
     }
 }
 
-template <typename T, bool ROWS, int LOGN>
-__device__ __forceinline__ typename Cx<T>::type *derive_n(T *P, typename Cx<T>::type *A, int logL, int ld,
-                                                          const typename Cx<T>::type *tw, const T *kn)
+template <typename T, bool ROWS, int LOGN, typename Next>
+__device__ __forceinline__ void derive_n(const T *P, typename Cx<T>::type *A, int logL, int ld,
+                                         const typename Cx<T>::type *tw, const T *kn, Next next)
 {
-    using C = typename Cx<T>::type;
-    constexpr int LOGR = pass_log(LOGN, 0, kMaxPassLog<T>);
-    C *B = reinterpret_cast<C *>(P);
     const int S = (1 << logL) + (1 << logL) / 2;
-    fft_first_pass<T, LOGN, ROWS>(P, A, logL, ld);
+    first_pass<T, LOGN, ROWS>(P, A, logL, ld, tw);
     __syncthreads();
-    C *r1 = Passes<T, LOGN, LOGR, false>::run(A, B, S, ld, tw + ((1 << LOGR) - 1), kn);
-    return Passes<T, LOGN, 0, true>::run(r1, r1 == A ? B : A, S, ld, tw, kn);
+    next();
+    Passes<T, LOGN, 0, false>::inner(A, S, ld, tw + (((1 << outer_log(LOGN, 0, kMaxPassLog<T>)) - 1)
+                                                    << (LOGN - outer_log(LOGN, 0, kMaxPassLog<T>))), kn);
+    outer_pass<T, LOGN, 0, false>(A, S, ld, tw);
+    __syncthreads();
 }
 
 // Spectral derivative of the staged lines: z = plane0 + i plane1 (and the plane-2
 // pairs), conj(FFT(conj(i k/N * FFT(z)))), for N = 2^logN, 2 <= N <= 2048.  The
-// first pass reads the planar staging P and writes A; P is scratch afterwards.
-// The returned buffer holds (D a, -D b) for each z = a + i b.
-template <typename T, bool ROWS>
-__device__ __forceinline__ typename Cx<T>::type *derive(T *P, typename Cx<T>::type *A, int logL, int logN, int ld,
-                                                        const typename Cx<T>::type *tw, const T *kn)
+// first pass reads the planar staging P, then next() runs (P is free); A then holds
+// (D a, -D b) for each z = a + i b.
+template <typename T, bool ROWS, typename Next>
+__device__ __forceinline__ void derive(const T *P, typename Cx<T>::type *A, int logL, int logN, int ld,
+                                       const typename Cx<T>::type *tw, const T *kn, Next next)
 {
     switch (logN) {
-    case 1: return derive_n<T, ROWS, 1>(P, A, logL, ld, tw, kn);
-    case 2: return derive_n<T, ROWS, 2>(P, A, logL, ld, tw, kn);
-    case 3: return derive_n<T, ROWS, 3>(P, A, logL, ld, tw, kn);
-    case 4: return derive_n<T, ROWS, 4>(P, A, logL, ld, tw, kn);
-    case 5: return derive_n<T, ROWS, 5>(P, A, logL, ld, tw, kn);
-    case 6: return derive_n<T, ROWS, 6>(P, A, logL, ld, tw, kn);
-    case 7: return derive_n<T, ROWS, 7>(P, A, logL, ld, tw, kn);
-    case 8: return derive_n<T, ROWS, 8>(P, A, logL, ld, tw, kn);
-    case 9: return derive_n<T, ROWS, 9>(P, A, logL, ld, tw, kn);
-    case 10: return derive_n<T, ROWS, 10>(P, A, logL, ld, tw, kn);
-    default: return derive_n<T, ROWS, 11>(P, A, logL, ld, tw, kn);
+    case 1: return derive_n<T, ROWS, 1>(P, A, logL, ld, tw, kn, next);
+    case 2: return derive_n<T, ROWS, 2>(P, A, logL, ld, tw, kn, next);
+    case 3: return derive_n<T, ROWS, 3>(P, A, logL, ld, tw, kn, next);
+    case 4: return derive_n<T, ROWS, 4>(P, A, logL, ld, tw, kn, next);
+    case 5: return derive_n<T, ROWS, 5>(P, A, logL, ld, tw, kn, next);
+    case 6: return derive_n<T, ROWS, 6>(P, A, logL, ld, tw, kn, next);
+    case 7: return derive_n<T, ROWS, 7>(P, A, logL, ld, tw, kn, next);
+    case 8: return derive_n<T, ROWS, 8>(P, A, logL, ld, tw, kn, next);
+    case 9: return derive_n<T, ROWS, 9>(P, A, logL, ld, tw, kn, next);
+    case 10: return derive_n<T, ROWS, 10>(P, A, logL, ld, tw, kn, next);
+    default: return derive_n<T, ROWS, 11>(P, A, logL, ld, tw, kn, next);
     }
 }
 
@@ -419,26 +431,23 @@ __device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_gr
 template <typename T, int VB>
 __device__ __forceinline__ void stage_copies(const SpecParams<T> &p, T *P, int kind, int level, int idx)
 {
-    constexpr int V = VB / (int)sizeof(T);            // values per copy
+    constexpr int kLogV = VB == (int)sizeof(T) ? 0 : (VB == 2 * (int)sizeof(T) ? 1 : 2);   // log2 of the values per copy
     if (kind == 0 && level < p.nz - 1) {
-        const int logn = p.logrx + p.lognx;
-        const int64_t base = (int64_t)level * p.nx * p.ny + ((int64_t)idx << logn);
-        const int per = (1 << logn) / V;
-        for (int c = threadIdx.x; c < 3 * per; c += kSpecThreads) {
-            const int f = c / per, q = c - f * per;
+        const int logn = p.logrx + p.lognx, logper = logn - kLogV;      // every count is a power of two
+        const int base = level * p.nx * p.ny + (idx << logn);
+        for (int c = threadIdx.x; c < 3 << logper; c += kSpecThreads) {
+            const int f = c >> logper, q = (c & ((1 << logper) - 1)) << kLogV;
             const T *src = f == 0 ? p.txx : (f == 1 ? p.txy : p.txz);
-            cp_async<VB>(P + ((int64_t)f << logn) + q * V, src + base + q * V);
+            cp_async<VB>(P + (f << logn) + q, src + base + q);
         }
     } else if (kind == 1 && level < p.nz - 1) {
-        const int logn = p.logny + p.logwy;
-        const int64_t base = (int64_t)level * p.nx * p.ny + ((int64_t)idx << p.logwy);
-        const int per_row = (1 << p.logwy) / V;
-        const int per = per_row << p.logny;
-        for (int c = threadIdx.x; c < 3 * per; c += kSpecThreads) {
-            const int f = c / per, q = c - f * per;
-            const int j = q / per_row, cc = q - j * per_row;
+        const int logn = p.logny + p.logwy, logper = logn - kLogV;
+        const int base = level * p.nx * p.ny + (idx << p.logwy);
+        for (int c = threadIdx.x; c < 3 << logper; c += kSpecThreads) {
+            const int f = c >> logper, q = (c & ((1 << logper) - 1)) << kLogV;
+            const int j = q >> p.logwy, cc = q & ((1 << p.logwy) - 1);
             const T *src = f == 0 ? p.txy : (f == 1 ? p.tyy : p.tyz);
-            cp_async<VB>(P + ((int64_t)f << logn) + (j << p.logwy) + cc * V, src + base + (int64_t)j * p.nx + cc * V);
+            cp_async<VB>(P + (f << logn) + q, src + base + (j << p.lognx) + cc);
         }
     }
 }
@@ -472,16 +481,16 @@ __device__ void stage_unit(const SpecParams<T> &p, T *P, int kind, int level, in
 
 // Row unit on level k, rows j0 .. j0 + rx - 1, whose input lines are staged in
 // P: d_x of txx, txy (sequences s < rx) and txz (rows 2q, 2q + 1 in rx + q),
-// plus the vertical terms -> the partial forcing in f.  P is scratch afterwards.
-template <typename T>
-__device__ void row_unit(const SpecParams<T> &p, T *P, typename Cx<T>::type *A, int k, int j0)
+// plus the vertical terms -> the partial forcing in f.
+template <typename T, typename Next>
+__device__ void row_unit(const SpecParams<T> &p, const T *P, typename Cx<T>::type *A, int k, int j0, Next next)
 {
     using C = typename Cx<T>::type;
     const int rx = 1 << p.logrx;
     const int n = rx << p.lognx;
-    const int64_t plane = (int64_t)p.nx * p.ny;
-    const int64_t base = (int64_t)k * plane + (int64_t)j0 * p.nx;
+    const int plane = p.nx * p.ny, base = k * plane + j0 * p.nx;
     if (k == p.nz - 1) {                    // ghost uv level / lid: f = 0
+        next();
         for (int e = threadIdx.x; e < n; e += kSpecThreads) {
             p.fx[base + e] = T(0);
             p.fy[base + e] = T(0);
@@ -490,11 +499,12 @@ __device__ void row_unit(const SpecParams<T> &p, T *P, typename Cx<T>::type *A, 
         return;
     }
     const int ld = p.ldx;
-    const C *R = derive<T, true>(P, A, p.logrx, p.lognx, ld, p.twx, p.knx);
+    derive<T, true>(P, A, p.logrx, p.lognx, ld, p.twx, p.knx, next);
+    const C *const R = A;
 #pragma unroll 4
     for (int e = threadIdx.x; e < n; e += kSpecThreads) {
         const int r = e >> p.lognx, i = e & (p.nx - 1);
-        const int64_t o = base + e;
+        const int o = base + e;
         const T xz0 = __ldg(p.txz + o), xz1 = __ldg(p.txz + o + plane);
         const T yz0 = __ldg(p.tyz + o), yz1 = __ldg(p.tyz + o + plane);
         const T zz0 = __ldg(p.tzz + o), zzm = k > 0 ? __ldg(p.tzz + o - plane) : T(0);
@@ -531,23 +541,28 @@ __device__ bool wait_level(const unsigned int *ctr, unsigned int target, int *st
 // Column unit on level k, columns i0 .. i0 + wy - 1, staged in P: d_y of txy, tyy
 // (sequences c < wy) and tyz (columns 2q, 2q + 1 in wy + q), subtracted from f
 // once every row unit of level k has written its partial forcing.
-template <typename T>
-__device__ void column_unit(const SpecParams<T> &p, T *P, typename Cx<T>::type *A, int k, int i0, int *s_go)
+template <typename T, typename Next>
+__device__ void column_unit(const SpecParams<T> &p, const T *P, typename Cx<T>::type *A, int k, int i0, int *s_go,
+                            Next next)
 {
     using C = typename Cx<T>::type;
-    if (k == p.nz - 1) return;              // f stays 0 there (written by the row units)
+    if (k == p.nz - 1) {                    // f stays 0 there (written by the row units)
+        next();
+        return;
+    }
     const int wy = 1 << p.logwy;
     const int n = wy << p.logny;
-    const int64_t base = (int64_t)k * p.nx * p.ny + i0;
+    const int base = k * p.nx * p.ny + i0;
     const int ld = p.ldy;
-    const C *R = derive<T, false>(P, A, p.logwy, p.logny, ld, p.twy, p.kny);
+    derive<T, false>(P, A, p.logwy, p.logny, ld, p.twy, p.kny, next);
+    const C *const R = A;
     if (threadIdx.x == 0) *s_go = wait_level(p.ctr + 2 + k, (unsigned)p.xpl, p.status) ? 1 : 0;
     __syncthreads();
     if (!*s_go) return;                     // gave up waiting: skipped, the status says so
 #pragma unroll 4
     for (int e = threadIdx.x; e < n; e += kSpecThreads) {
         const int j = e >> p.logwy, c = e & (wy - 1);
-        const int64_t o = base + (int64_t)j * p.nx + c;
+        const int o = base + (j << p.lognx) + c;
         const T fx0 = __ldcg(p.fx + o), fy0 = __ldcg(p.fy + o), fz0 = __ldcg(p.fz + o);
         const C d = R[c * ld + sk(j)];                      // (d_y txy, -d_y tyy)
         const C dd = R[(wy + (c >> 1)) * ld + sk(j)];
@@ -601,42 +616,41 @@ __device__ __forceinline__ void claim(const SpecParams<T> &p, int *slot)
 }
 
 // Persistent loop: each block holds the unit it works on and the next one, whose
-// input lines stream into the other staging buffer meanwhile.  A column unit
-// waits only for the row units of its level, which hold smaller tickets; the
-// unfinished unit with the smallest ticket can always proceed, so the loop
-// ends.  Shared memory: staging buffers P0, P1 and the FFT buffer A, each buf
-// complex elements.
+// input lines stream into the staging buffer as soon as the unit's first pass has
+// read its own from there.  A column unit waits only for the row units of its level,
+// which hold smaller tickets; the unfinished unit with the smallest ticket can
+// always proceed, so the loop ends.  Shared memory: the FFT buffer A and the staging
+// buffer P (a second one would leave the tables and the epilogue's loads a few KB of
+// L1).
 template <typename T>
-__global__ void __launch_bounds__(kSpecThreads, sizeof(T) == 4 ? 3 : 2) k_spectral(SpecParams<T> p)
+__global__ void __launch_bounds__(kSpecThreads, sizeof(T) == 4 ? 4 : 2) k_spectral(SpecParams<T> p)
 {
     using C = typename Cx<T>::type;
     extern __shared__ __align__(16) unsigned char spec_smem[];
     C *A = reinterpret_cast<C *>(spec_smem);
-    T *const P0 = reinterpret_cast<T *>(A + p.buf);
-    T *const P1 = reinterpret_cast<T *>(A + 2 * p.buf);
+    T *const P = reinterpret_cast<T *>(A + p.buf);
     __shared__ int s_u[2][3];
     __shared__ int s_go, s_last;
     int cur = 0;
     if (threadIdx.x == 0) claim(p, s_u[0]);
     __syncthreads();
-    stage_unit<T>(p, P0, s_u[0][0], s_u[0][1], s_u[0][2]);
+    stage_unit<T>(p, P, s_u[0][0], s_u[0][1], s_u[0][2]);
     for (;;) {
         const int kind = s_u[cur][0], level = s_u[cur][1], idx = s_u[cur][2];
         if (kind < 0) break;
         if (threadIdx.x == 0) claim(p, s_u[cur ^ 1]);
+        cp_async_wait<0>();                 // this unit's lines have landed
         __syncthreads();
-        stage_unit<T>(p, cur ? P0 : P1, s_u[cur ^ 1][0], s_u[cur ^ 1][1], s_u[cur ^ 1][2]);
-        cp_async_wait<1>();                 // this unit's lines have landed (the next unit's may not)
-        __syncthreads();
+        auto next = [&] { stage_unit<T>(p, P, s_u[cur ^ 1][0], s_u[cur ^ 1][1], s_u[cur ^ 1][2]); };
         if (kind == 0) {
-            row_unit<T>(p, cur ? P1 : P0, A, level, idx << p.logrx);
+            row_unit<T>(p, P, A, level, idx << p.logrx, next);
             __syncthreads();
             if (threadIdx.x == 0) {
                 __threadfence();
                 atomicAdd(p.ctr + 2 + level, 1u);
             }
         } else {
-            column_unit<T>(p, cur ? P1 : P0, A, level, idx << p.logwy, &s_go);
+            column_unit<T>(p, P, A, level, idx << p.logwy, &s_go, next);
             __syncthreads();
         }
         cur ^= 1;
@@ -685,24 +699,36 @@ int upload_tables(wmibm_handle *h, SpecState *s, cudaStream_t stream)
             free(hk);
             return set_error(nullptr, WMIBM_ENOMEM, "host memory for the spectral tables");
         }
-        // per-pass twiddles: pass (Ns, R) holds omega_N^(r jm N/(Ns R)) at (r - 1) Ns + jm
-        int at = 0;
-        for (int logNs = 0, logN = ilog2_exact(N); logNs < logN;) {
-            const int logR = pass_log(logN, logNs, kMaxPassLog<T>);
-            const int Ns = 1 << logNs, R = 1 << logR;
-            for (int r = 1; r < R; ++r)
-                for (int jm = 0; jm < Ns; ++jm) {
-                    const double a = 2.0 * M_PI * (double)r * (double)jm / (double)(Ns * R);
+        // twiddles of the outer passes: on blocks of M elements, omega_M^(j q) at (q - 1) M / R + j
+        const int logN = ilog2_exact(N), maxlog = kMaxPassLog<T>;
+        int at = 0, used = 0;
+        for (int logR; (logR = outer_log(logN, used, maxlog)) > 0; used += logR) {
+            const int M = N >> used, R = 1 << logR, step = M / R;
+            for (int q = 1; q < R; ++q)
+                for (int j = 0; j < step; ++j) {
+                    const double a = 2.0 * M_PI * (double)j * (double)q / (double)M;
                     ht[at].x = (T)cos(a);
                     ht[at].y = (T)(-sin(a));
                     ++at;
                 }
-            logNs += logR;
         }
-        for (int m = 0; m < N; ++m) {
-            // wavenumber of bin m: m below N/2, m - N above, 0 for the Nyquist bin
+        for (int e = 0; e < N; ++e) {
+            // the bin that the forward transform leaves at element e: the passes' digits of e, the first one's
+            // (the most significant) counting least
+            int m = 0, left = e, size = N, weight = 1;
+            for (int u = 0; size > 1;) {
+                int logR = outer_log(logN, u, maxlog);
+                if (logR == 0) logR = ilog2_exact(size);    // the middle pass
+                const int R = 1 << logR, step = size / R;
+                m += weight * (left / step);
+                left %= step;
+                weight *= R;
+                size = step;
+                u += logR;
+            }
+            // its wavenumber: m below N/2, m - N above, 0 for the Nyquist bin
             const int mm = (2 * m < N) ? m : (2 * m == N ? 0 : m - N);
-            hk[m] = (T)(2.0 * M_PI * (double)mm / len[d] / (double)N);
+            hk[e] = (T)(2.0 * M_PI * (double)mm / len[d] / (double)N);
         }
         cudaError_t e = dev_alloc(tw[d], sizeof(C) * N);
         if (e == cudaSuccess) e = dev_alloc(kn[d], sizeof(T) * N);
@@ -752,7 +778,7 @@ int launch_spectral(wmibm_handle *h, const void *const tau[6], void *fx, void *f
     p.ldx = s->ldx; p.ldy = s->ldy;
     p.kc = s->kc; p.nchunks = s->nchunks; p.xpl = s->xpl; p.ypl = s->ypl;
     p.total = s->total;
-    p.buf = (int)(s->smem / (3 * sizeof(typename Cx<T>::type)));
+    p.buf = (int)s->buf;
     p.rdz = (T)(1.0 / h->dz);
     // 16-byte copies when every staged line segment starts on a 16-byte boundary
     bool v16 = (h->nx * sizeof(T)) % 16 == 0 && (s->wy * sizeof(T)) % 16 == 0;
@@ -785,15 +811,16 @@ int spectral_setup(wmibm_handle *h, cudaStream_t stream)
     const size_t cs = f64 ? 16 : 8;
     const int budget = f64 ? kSpecBudget / 2 : kSpecBudget;
     // rows per row unit: even power of two dividing ny, 1.5 rx (nx + 1) within the budget
-    s->ldx = h->nx + (h->nx >> 5) + 1;       // skewed sequence (e + e/32) plus one: odd-ish bank offset
+    s->ldx = h->nx + (h->nx >> 4) + 1;       // skewed sequence (e + e/16) plus one: odd-ish bank offset
     s->rx = 2;
     while (s->rx * 2 <= h->ny && 3 * (s->rx * 2) / 2 * s->ldx <= budget) s->rx *= 2;
-    s->ldy = h->ny + (h->ny >> 5) + 1;
+    s->ldy = h->ny + (h->ny >> 4) + 1;
     s->wy = 2;
     while (s->wy * 2 <= h->nx && 3 * (s->wy * 2) / 2 * s->ldy <= budget) s->wy *= 2;
     const int64_t ex = (int64_t)3 * s->rx / 2 * s->ldx, ey = (int64_t)3 * s->wy / 2 * s->ldy;
-    const int64_t buf = ((ex > ey ? ex : ey) + 1) & ~(int64_t)1;    // even: 16-byte aligned buffers
-    s->smem = 3 * cs * (size_t)buf;
+    s->buf = ((ex > ey ? ex : ey) + 1) & ~(int64_t)1;               // even: 16-byte aligned buffers
+    const int64_t px = (int64_t)3 * s->rx * h->nx, py = (int64_t)3 * s->wy * h->ny;
+    s->smem = cs * (size_t)s->buf + (cs / 2) * (size_t)(px > py ? px : py);
     s->xpl = h->ny / s->rx;
     s->ypl = h->nx / s->wy;
     const double level_bytes = 9.0 * (double)h->nx * (double)h->ny * (double)elem_size(h->dtype);
