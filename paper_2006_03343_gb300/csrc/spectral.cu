@@ -86,6 +86,7 @@ struct SpecParams {
     int32_t kc, nchunks, xpl, ypl;
     int64_t total;
     int32_t buf;              // complex elements of the FFT buffer
+    int32_t wide;             // 16-byte runs in the epilogues as well (every run of the forcing 16-byte aligned)
     int32_t v16;              // stage with 16-byte copies (every staged segment 16-byte aligned)
     T rdz;
 };
@@ -479,16 +480,73 @@ __device__ void stage_unit(const SpecParams<T> &p, T *P, int kind, int level, in
     }
 }
 
+// V consecutive values of a global array (V > 1: 16-byte aligned); L2: past L1.
+template <typename T, int V>
+struct Run {
+    T v[V];
+};
+template <bool L2, typename T>
+__device__ __forceinline__ T ld(const T *p) { return L2 ? __ldcg(p) : __ldg(p); }
+template <int V, bool L2, typename T>
+__device__ __forceinline__ Run<T, V> ld_run(const T *p)
+{
+    Run<T, V> r;
+    if constexpr (V == 4) {
+        const float4 a = ld<L2>(reinterpret_cast<const float4 *>(p));
+        r.v[0] = a.x; r.v[1] = a.y; r.v[2] = a.z; r.v[3] = a.w;
+    } else if constexpr (V == 2) {
+        const double2 a = ld<L2>(reinterpret_cast<const double2 *>(p));
+        r.v[0] = a.x; r.v[1] = a.y;
+    } else {
+        r.v[0] = ld<L2>(p);
+    }
+    return r;
+}
+template <int V, typename T>
+__device__ __forceinline__ void st_run(T *p, const Run<T, V> &r)
+{
+    if constexpr (V == 4) *reinterpret_cast<float4 *>(p) = make_float4(r.v[0], r.v[1], r.v[2], r.v[3]);
+    else if constexpr (V == 2) *reinterpret_cast<double2 *>(p) = make_double2(r.v[0], r.v[1]);
+    else *p = r.v[0];
+}
+
+// The row unit's forcing from its derivatives R and the vertical terms.
+template <typename T, int V>
+__device__ __forceinline__ void row_forcing(const SpecParams<T> &p, const typename Cx<T>::type *R, int k, int base)
+{
+    using C = typename Cx<T>::type;
+    const int rx = 1 << p.logrx, n = rx << p.lognx, plane = p.nx * p.ny, ld = p.ldx;
+#pragma unroll 2
+    for (int e = threadIdx.x * V; e < n; e += kSpecThreads * V) {
+        const int r = e >> p.lognx, i = e & (p.nx - 1), o = base + e;
+        const Run<T, V> xz0 = ld_run<V, false>(p.txz + o), xz1 = ld_run<V, false>(p.txz + o + plane);
+        const Run<T, V> yz0 = ld_run<V, false>(p.tyz + o), yz1 = ld_run<V, false>(p.tyz + o + plane);
+        const Run<T, V> zz0 = ld_run<V, false>(p.tzz + o);
+        Run<T, V> zzm = zz0, fx, fy, fz;
+        if (k > 0) zzm = ld_run<V, false>(p.tzz + o - plane);
+        // V divides 16: the skew is the same for all of a run
+        const C *const d = R + r * ld + sk(i), *const dd = R + (rx + (r >> 1)) * ld + sk(i);
+#pragma unroll
+        for (int q = 0; q < V; ++q) {
+            const C a = d[q], b = dd[q];                        // (d_x txx, -d_x txy), d_x txz of two rows
+            const T dxz = (r & 1) ? -b.y : b.x;
+            fx.v[q] = -(a.x + (xz1.v[q] - xz0.v[q]) * p.rdz);
+            fy.v[q] = -(-a.y + (yz1.v[q] - yz0.v[q]) * p.rdz);
+            fz.v[q] = (k == 0) ? T(0) : -(dxz + (zz0.v[q] - zzm.v[q]) * p.rdz);
+        }
+        st_run(p.fx + o, fx);
+        st_run(p.fy + o, fy);
+        st_run(p.fz + o, fz);
+    }
+}
+
 // Row unit on level k, rows j0 .. j0 + rx - 1, whose input lines are staged in
 // P: d_x of txx, txy (sequences s < rx) and txz (rows 2q, 2q + 1 in rx + q),
 // plus the vertical terms -> the partial forcing in f.
 template <typename T, typename Next>
 __device__ void row_unit(const SpecParams<T> &p, const T *P, typename Cx<T>::type *A, int k, int j0, Next next)
 {
-    using C = typename Cx<T>::type;
-    const int rx = 1 << p.logrx;
-    const int n = rx << p.lognx;
-    const int plane = p.nx * p.ny, base = k * plane + j0 * p.nx;
+    const int n = 1 << (p.logrx + p.lognx), base = k * p.nx * p.ny + j0 * p.nx;
     if (k == p.nz - 1) {                    // ghost uv level / lid: f = 0
         next();
         for (int e = threadIdx.x; e < n; e += kSpecThreads) {
@@ -498,23 +556,9 @@ __device__ void row_unit(const SpecParams<T> &p, const T *P, typename Cx<T>::typ
         }
         return;
     }
-    const int ld = p.ldx;
-    derive<T, true>(P, A, p.logrx, p.lognx, ld, p.twx, p.knx, next);
-    const C *const R = A;
-#pragma unroll 4
-    for (int e = threadIdx.x; e < n; e += kSpecThreads) {
-        const int r = e >> p.lognx, i = e & (p.nx - 1);
-        const int o = base + e;
-        const T xz0 = __ldg(p.txz + o), xz1 = __ldg(p.txz + o + plane);
-        const T yz0 = __ldg(p.tyz + o), yz1 = __ldg(p.tyz + o + plane);
-        const T zz0 = __ldg(p.tzz + o), zzm = k > 0 ? __ldg(p.tzz + o - plane) : T(0);
-        const C d = R[r * ld + sk(i)];                      // (d_x txx, -d_x txy)
-        const C dd = R[(rx + (r >> 1)) * ld + sk(i)];
-        const T dxz = (r & 1) ? -dd.y : dd.x;               // d_x txz
-        p.fx[o] = -(d.x + (xz1 - xz0) * p.rdz);
-        p.fy[o] = -(-d.y + (yz1 - yz0) * p.rdz);
-        p.fz[o] = (k == 0) ? T(0) : -(dxz + (zz0 - zzm) * p.rdz);
-    }
+    derive<T, true>(P, A, p.logrx, p.lognx, p.ldx, p.twx, p.knx, next);
+    if (p.wide) row_forcing<T, 16 / (int)sizeof(T)>(p, A, k, base);
+    else row_forcing<T, 1>(p, A, k, base);
 }
 
 // Waits until *ctr >= target (acquire, GPU scope); bounded by kWaitLimitNs.
@@ -538,6 +582,31 @@ __device__ bool wait_level(const unsigned int *ctr, unsigned int target, int *st
     }
 }
 
+// Subtracts the column unit's derivatives R from the partial forcing.
+template <typename T, int V>
+__device__ __forceinline__ void column_forcing(const SpecParams<T> &p, const typename Cx<T>::type *R, int k, int base)
+{
+    using C = typename Cx<T>::type;
+    const int wy = 1 << p.logwy, n = wy << p.logny, ld = p.ldy;
+#pragma unroll 2
+    for (int e = threadIdx.x * V; e < n; e += kSpecThreads * V) {
+        const int j = e >> p.logwy, c = e & (wy - 1), o = base + (j << p.lognx) + c;
+        Run<T, V> fx = ld_run<V, true>(p.fx + o), fy = ld_run<V, true>(p.fy + o), fz = ld_run<V, true>(p.fz + o);
+#pragma unroll
+        for (int q = 0; q < V; ++q) {
+            const C d = R[(c + q) * ld + sk(j)];                // (d_y txy, -d_y tyy)
+            const C dd = R[(wy + ((c + q) >> 1)) * ld + sk(j)];
+            const T dyz = ((c + q) & 1) ? -dd.y : dd.x;         // d_y tyz
+            fx.v[q] -= d.x;
+            fy.v[q] += d.y;
+            fz.v[q] -= dyz;
+        }
+        st_run(p.fx + o, fx);
+        st_run(p.fy + o, fy);
+        if (k > 0) st_run(p.fz + o, fz);
+    }
+}
+
 // Column unit on level k, columns i0 .. i0 + wy - 1, staged in P: d_y of txy, tyy
 // (sequences c < wy) and tyz (columns 2q, 2q + 1 in wy + q), subtracted from f
 // once every row unit of level k has written its partial forcing.
@@ -550,27 +619,13 @@ __device__ void column_unit(const SpecParams<T> &p, const T *P, typename Cx<T>::
         next();
         return;
     }
-    const int wy = 1 << p.logwy;
-    const int n = wy << p.logny;
     const int base = k * p.nx * p.ny + i0;
-    const int ld = p.ldy;
-    derive<T, false>(P, A, p.logwy, p.logny, ld, p.twy, p.kny, next);
-    const C *const R = A;
+    derive<T, false>(P, A, p.logwy, p.logny, p.ldy, p.twy, p.kny, next);
     if (threadIdx.x == 0) *s_go = wait_level(p.ctr + 2 + k, (unsigned)p.xpl, p.status) ? 1 : 0;
     __syncthreads();
     if (!*s_go) return;                     // gave up waiting: skipped, the status says so
-#pragma unroll 4
-    for (int e = threadIdx.x; e < n; e += kSpecThreads) {
-        const int j = e >> p.logwy, c = e & (wy - 1);
-        const int o = base + (j << p.lognx) + c;
-        const T fx0 = __ldcg(p.fx + o), fy0 = __ldcg(p.fy + o), fz0 = __ldcg(p.fz + o);
-        const C d = R[c * ld + sk(j)];                      // (d_y txy, -d_y tyy)
-        const C dd = R[(wy + (c >> 1)) * ld + sk(j)];
-        const T dyz = (c & 1) ? -dd.y : dd.x;               // d_y tyz
-        p.fx[o] = fx0 - d.x;
-        p.fy[o] = fy0 + d.y;
-        if (k > 0) p.fz[o] = fz0 - dyz;
-    }
+    if (p.wide) column_forcing<T, 16 / (int)sizeof(T)>(p, A, k, base);
+    else column_forcing<T, 1>(p, A, k, base);
 }
 
 // Unit u of the dispense order -> kind (0 row, 1 column), level, index within the level.
@@ -784,6 +839,8 @@ int launch_spectral(wmibm_handle *h, const void *const tau[6], void *fx, void *f
     bool v16 = (h->nx * sizeof(T)) % 16 == 0 && (s->wy * sizeof(T)) % 16 == 0;
     for (int c = 0; c < 6; ++c) v16 = v16 && ((uintptr_t)tau[c] & 15u) == 0;
     p.v16 = v16 ? 1 : 0;
+    for (const void *q : {fx, fy, fz}) v16 = v16 && ((uintptr_t)q & 15u) == 0;
+    p.wide = v16 ? 1 : 0;
     return run_spectral<T>(h, p, s, stream);
 }
 
