@@ -39,7 +39,10 @@ namespace wmibm {
 constexpr int kSpecMaxLog = 11;         // lines of up to 2048 points (FP32; 1024 for FP64)
 constexpr int kSpecThreads = 192;
 constexpr int kSpecBudget = 3300;       // complex elements per shared buffer aimed at (FP32; half for FP64)
-constexpr double kSpecChunkBytes = 24.0 * 1024 * 1024;   // L2 footprint of one chunk of levels
+// L2 footprint of one chunk of levels: below it the column units wait for their row
+// units, above it their second reads miss L2 (hill, FP32: 12 / 24 / 32 / 48 / 72 MB: 967 /
+// 742 / 761 / 789 / 797 us).
+constexpr double kSpecChunkBytes = 24.0 * 1024 * 1024;
 
 struct SpecState {
     int lognx, logny;
@@ -670,6 +673,16 @@ __device__ __forceinline__ void claim(const SpecParams<T> &p, int *slot)
     slot[2] = idx;
 }
 
+// Bound, FP32: shared-memory accesses, issue and the barriers between passes (hill
+// 512 x 256 x 256: 722 us against 178 us for its bytes at the copy peak; 256 x 128 x
+// 128 77 us, 64^3 14.7 us); a Stockham pair of transforms with two more buffers, three
+// blocks of 256 threads per SM, took 765, 93 and 17 us.  FP64: the FP64 pipe, about 150
+// operations a point, 1.09 ms of 1.20 ms on 256 x 128 x 128.  192 threads divide the
+// passes of the common tiles evenly (six sequences of 512 points are 192 butterflies
+// of radix 16): four blocks of 192 per SM 742 us, of 256 788, three of 256 779, five of
+// 192 820, eight of 96 1070 (before the 16-byte epilogues).  FP64: radix 16 or three
+// blocks per SM 1211 and 1231 us against 1202.
+//
 // Persistent loop: each block holds the unit it works on and the next one, whose
 // input lines stream into the staging buffer as soon as the unit's first pass has
 // read its own from there.  A column unit waits only for the row units of its level,

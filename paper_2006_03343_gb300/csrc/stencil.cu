@@ -1,9 +1,10 @@
-// Bulk-copy (TMA) pipelined stencil for f = -div(tau) (Eq. 2, Eq. 18, Eqs. 15-16
-// of Liu & Stevens, arXiv:2006.03343), the persistent wall-model kernel
-// (Sec. 3.3), and the body mask (Eq. 27), for one terrain or for a batch of
-// terrains ("members") of uneven grid sizes in the same launches.
+// The stencil for f = -div(tau) (Eq. 2, Eq. 18, Eqs. 15-16 of Liu & Stevens,
+// arXiv:2006.03343) in two forms, by direct loads (k_direct, untuned launches) and as
+// a bulk-copy (TMA) pipeline (k_stencil, where the tuning asks for it), the
+// persistent wall-model kernel (Sec. 3.3), and the body mask (Eq. 27), for one terrain
+// or for a batch of terrains ("members") of uneven grid sizes in the same launches.
 //
-// Stencil: every member's grid is cut into strips of TY full x-rows
+// Pipelined stencil: every member's grid is cut into strips of TY full x-rows
 // (j0 .. j0+TY-1); the (member, strip, level) units are split evenly over a
 // persistent grid.  Per block, lane 0 of warp 0 is the producer: it issues 1D
 // bulk copies of the rows a stage needs into a ring of S shared-memory stages
