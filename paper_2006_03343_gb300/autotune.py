@@ -45,8 +45,9 @@ WALL_WARPS_IN_BLOCK = (1, 2, 3)     # wall warps beside the producer and consume
 DYN_CHUNKS = (0, 16)                # units per take of the dynamic dispensing (0: a fixed share per block)
 WALL_GRIDS = (0, 2)                 # blocks per SM of the separate wall kernel (0: as many as fit)
 
-# the untuned form: the wall kernel and the direct-load stencil; tried beside the candidates' shapes
-DEFAULT_FORM = "direct"
+# the untuned form, the wall kernel and the direct-load stencil, tried beside the candidates' shapes
+# (a batch counts it among its two-launch forms)
+DIRECT, BATCH_DIRECT = {"force_path": 2}, {"force_path": 0}
 FORM_NAMES = {1: "single_launch", 2: "direct", 3: "two_launch", 4: "dedicated_wall_blocks", 5: "interleaved",
               6: "wall_warps"}
 
@@ -244,7 +245,7 @@ def tune(handle, fields, reps: int = 9, use_cache: bool = True, budget_s: float 
     best_form = {}                          # fastest (ms, tuning) per form
     tried = 0
     t_start = time.perf_counter()
-    for cand in [{}] + candidates(handle):
+    for cand in [DIRECT] + candidates(handle):
         if time.perf_counter() - t_start > budget_s:
             break
         try:
@@ -255,7 +256,7 @@ def tune(handle, fields, reps: int = 9, use_cache: bool = True, budget_s: float 
         if verbose:
             print(f"  {ms * 1e3:8.1f} us  {cand}")
         timed.append((ms, cand))
-        form = FORM_NAMES[cand.get("force_path", 1)] if cand else DEFAULT_FORM
+        form = FORM_NAMES[cand.get("force_path", 1)]
         if form not in best_form or ms < best_form[form][0]:
             best_form[form] = (ms, cand)
     if not timed:
@@ -267,7 +268,7 @@ def tune(handle, fields, reps: int = 9, use_cache: bool = True, budget_s: float 
 
     def rank(item):
         ms, cand = item
-        if two is not None and cand and cand.get("force_path") != 3 and ms > (1.0 - SINGLE_MARGIN) * two[0]:
+        if two is not None and cand.get("force_path") not in (2, 3) and ms > (1.0 - SINGLE_MARGIN) * two[0]:
             return (1, ms)
         return (0, ms)
 
@@ -316,7 +317,7 @@ def tune_batch(batch, stats=None, reps: int = 7, use_cache: bool = True, budget_
     best_form = {}
     tried = 0
     t_start = time.perf_counter()
-    for cand in [{}] + batch_candidates(batch):
+    for cand in [BATCH_DIRECT] + batch_candidates(batch):
         if time.perf_counter() - t_start > budget_s:
             break
         try:
@@ -328,7 +329,7 @@ def tune_batch(batch, stats=None, reps: int = 7, use_cache: bool = True, budget_
         if verbose:
             print(f"  {ms * 1e3:8.1f} us  {cand}")
         timed.append((ms, cand))
-        form = FORM_NAMES[cand["force_path"]] if cand else DEFAULT_FORM
+        form = FORM_NAMES[cand["force_path"] or 3]
         if form not in best_form or ms < best_form[form][0]:
             best_form[form] = (ms, cand)
     if not timed:
