@@ -256,22 +256,58 @@ __device__ __forceinline__ void stats_combine(T *dst, const T *src)
     }
 }
 
+// Reduces acc over the warp; lane l returns the total of value l / 4.  Each exchange
+// halves the values that a lane carries on (4 + 2 + 1 + 1 + 1 steps of one value
+// instead of 8 x 5: in FP64 a step costs its SM 16 cycles of the pipe a warp), so
+// lanes that keep a sum and lanes that keep a minimum (of -|U_r| for the maximum)
+// meet in one step and choose.
+template <typename T>
+__device__ __forceinline__ T stats_warp_reduce(const T acc[kStatVals])
+{
+    constexpr unsigned all = 0xffffffffu;
+    const int lane = threadIdx.x & 31;
+    const bool band = lane & 16, extreme = lane & 8, second = lane & 4;
+    T x[4], y[2];
+    for (int s = 0; s < 4; ++s) {
+        const T a = s == 3 ? -acc[3] : acc[s], b = s == 3 ? -acc[7] : acc[4 + s];
+        const T own = band ? b : a, other = __shfl_xor_sync(all, band ? a : b, 16);
+        x[s] = s < 2 ? own + other : min(own, other);
+    }
+    for (int s = 0; s < 2; ++s) {
+        const T own = extreme ? x[2 + s] : x[s], other = __shfl_xor_sync(all, extreme ? x[s] : x[2 + s], 8);
+        y[s] = extreme ? min(own, other) : own + other;
+    }
+    T z = second ? y[1] : y[0];
+    T other = __shfl_xor_sync(all, second ? y[0] : y[1], 4);
+    z = extreme ? min(z, other) : z + other;
+    for (int o = 2; o > 0; o >>= 1) {
+        other = __shfl_xor_sync(all, z, o);
+        z = extreme ? min(z, other) : z + other;
+    }
+    return extreme && second ? -z : z;
+}
+
 // All threads of the block call this; thread 0 ends up with the block total.
 template <typename T>
 __device__ void stats_block_reduce(T acc[kStatVals], T (*smem)[kStatVals])
 {
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarps = (blockDim.x + 31) >> 5;
-    for (int b = 0; b < 2; ++b) {
-        acc[4 * b + 0] = warp_sum(acc[4 * b + 0]);
-        acc[4 * b + 1] = warp_sum(acc[4 * b + 1]);
-        acc[4 * b + 2] = warp_min(acc[4 * b + 2]);
-        acc[4 * b + 3] = warp_max(acc[4 * b + 3]);
-    }
-    if (lane == 0)
-        for (int s = 0; s < kStatVals; ++s) smem[warp][s] = acc[s];
+    const T z = stats_warp_reduce(acc);
+    if ((lane & 3) == 0) smem[warp][lane >> 2] = z;
     __syncthreads();
-    if (threadIdx.x == 0)
-        for (int w = 1; w < nwarps; ++w) stats_combine(acc, smem[w]);
+    if (warp == 0) {
+        if (nwarps > 1 && lane < kStatVals) {
+            T v = smem[0][lane];
+            for (int w = 1; w < nwarps; ++w) {
+                const T o = smem[w][lane];
+                v = (lane & 3) < 2 ? v + o : ((lane & 3) == 2 ? min(v, o) : max(v, o));
+            }
+            smem[0][lane] = v;
+        }
+        __syncwarp();
+        if (lane == 0)
+            for (int s = 0; s < kStatVals; ++s) acc[s] = smem[0][s];
+    }
     __syncthreads();
 }
 

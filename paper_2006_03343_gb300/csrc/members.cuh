@@ -105,9 +105,10 @@ int batch_launch(wmibm_handle *h0, const Member<T> *dev_members, int nmembers, c
 
 bool stencil_config(const wmibm_handle *h, const void *const tau[6], void *const f[3], StencilConfig *out);
 
-// The direct-load stencil's tile of a member for vectors of v values: bx vectors by by rows, kc levels (0: chosen).
+// The direct-load stencil's tile of a member for vectors of v values: bx vectors by by rows, kc levels (0: chosen;
+// rows so that the grid has at least `blocks` blocks where that is possible).
 template <typename T>
-void direct_tile(Member<T> &m, int v, int bx, int by, int kc);
+void direct_tile(Member<T> &m, int v, int bx, int by, int kc, int blocks);
 
 template <typename T>
 bool whole_sectors(const Member<T> &m);
