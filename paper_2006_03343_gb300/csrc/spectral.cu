@@ -28,6 +28,7 @@
 // from L2 while DRAM streams each array once.  Row units never wait, and every
 // row unit a column unit depends on was dispensed earlier to a running block,
 // so the waits end whatever the grid size.
+#include <algorithm>
 #include <math.h>
 #include <stdlib.h>
 
@@ -886,7 +887,11 @@ int spectral_setup(wmibm_handle *h, cudaStream_t stream)
     while (s->rx * 2 <= h->ny && 3 * (s->rx * 2) / 2 * s->ldx <= budget) s->rx *= 2;
     s->ldy = h->ny + (h->ny >> 4) + 1;
     s->wy = 2;
-    while (s->wy * 2 <= h->nx && 3 * (s->wy * 2) / 2 * s->ldy <= budget) s->wy *= 2;
+    // FP32: at least a 32-byte sector of columns where shared memory has the room, whatever
+    // that leaves of the blocks per SM (columns of 512 points, 4 / 8 of them: 1024 x 512 x 18
+    // 332 / 292 us, 512 x 512 x 64 566 / 515; of 1024, 2 / 4 / 8: 512 x 1024 x 20 659 / 451 / 441)
+    auto room = [&](int wy) { return !f64 && wy <= 8 && (12 * (size_t)s->ldy + 12 * (size_t)h->ny) * wy <= 220 * 1024; };
+    while (s->wy * 2 <= h->nx && (3 * (s->wy * 2) / 2 * s->ldy <= budget || room(s->wy * 2))) s->wy *= 2;
     const int64_t ex = (int64_t)3 * s->rx / 2 * s->ldx, ey = (int64_t)3 * s->wy / 2 * s->ldy;
     s->buf = ((ex > ey ? ex : ey) + 1) & ~(int64_t)1;               // even: 16-byte aligned buffers
     const int64_t px = (int64_t)3 * s->rx * h->nx, py = (int64_t)3 * s->wy * h->ny;
@@ -895,7 +900,11 @@ int spectral_setup(wmibm_handle *h, cudaStream_t stream)
     s->ypl = h->nx / s->wy;
     const double level_bytes = 9.0 * (double)h->nx * (double)h->ny * (double)elem_size(h->dtype);
     s->kc = (int)(kSpecChunkBytes / level_bytes);
-    if (s->kc < 1) s->kc = 1;
+    const int resident = h->sm_count * std::min<int>(f64 ? 2 : 4, (int)(227 * 1024 / (s->smem + 1024)));
+    // and at least half the resident blocks' number of row units a chunk: the column units of
+    // a shorter one wait (1024 x 512 x 18 with chunks of one and two levels 378 and 335 us,
+    // 512 x 512 x 64 of two and three 638 and 569)
+    s->kc = std::max(s->kc, (resident / 2 + s->xpl - 1) / s->xpl);
     if (s->kc > h->nz) s->kc = h->nz;
     s->nchunks = (h->nz + s->kc - 1) / s->kc;
     s->total = (int64_t)h->nz * (s->xpl + s->ypl);
