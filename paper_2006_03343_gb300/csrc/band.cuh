@@ -122,6 +122,15 @@ __device__ __forceinline__ void band_fetch_shared(const typename RecOf<T>::type 
     band_gather<T, V>(ix, u, v, w, nx, ny, plane, b);
 }
 
+// A velocity value by an ordinary load: the body mask, or whatever the wall kernel waits
+// for, may write the velocity while the launch runs.
+template <typename V, typename T>
+__device__ __forceinline__ T gather_vel(const V *p, int64_t i)
+{
+    if constexpr (sizeof(V) == 2) return __bfloat162float(p[i]);
+    else return p[i];
+}
+
 // The 24 corner values of the node whose record unpacked to ix.
 template <typename T, typename V>
 __device__ __forceinline__ void band_gather(const int4 ix, const V *u, const V *v, const V *w, int32_t nx,
@@ -137,9 +146,9 @@ __device__ __forceinline__ void band_gather(const int4 ix, const V *u, const V *
 #pragma unroll
     for (int c = 0; c < 8; ++c) {
         const int32_t o = ((c & 1) ? di : 0) + ((c & 2) ? dj : 0) + ((c & 4) ? dk : 0);
-        b.cu[c] = load_vel<V, T>(pu, o);
-        b.cv[c] = load_vel<V, T>(pv, o);
-        b.cw[c] = load_vel<V, T>(pw, o);
+        b.cu[c] = gather_vel<V, T>(pu, o);
+        b.cv[c] = gather_vel<V, T>(pv, o);
+        b.cw[c] = gather_vel<V, T>(pw, o);
     }
 }
 
@@ -162,7 +171,7 @@ __device__ __forceinline__ BandOut<T> band_finish(const BandIn<T> &b, bool is_w,
     const T vc = trilinear8(b.cv, b.ax, b.ay, b.azu);
     const T wc = trilinear8(b.cw, b.ax, b.ay, b.azw);
     if (logz0) {
-        const T d = log_phi_c - __ldg(logz0 + b.idx);
+        const T d = log_phi_c - logz0[b.idx];
         C = kappa2 / (d * d);
     }
     const T un = uc * nxv + vc * nyv + wc * nzv;

@@ -913,19 +913,13 @@ __global__ void __launch_bounds__(256) k_wall(KParams<T> p)
     __shared__ T red[32][kStatVals];
     __shared__ bool s_last;
     const Member<T> &mm = p.one;
-    const VEL *u = reinterpret_cast<const VEL *>(mm.u), *v = reinterpret_cast<const VEL *>(mm.v),
-              *w = reinterpret_cast<const VEL *>(mm.w);
-    const T *logz0 = mm.logz0;
-    // wait for what is before in the stream (the pointers go through, so that no read-only
-    // load moves ahead of it), then let the stencil kernel, next in it, launch right away
-    asm volatile("griddepcontrol.wait;" : "+l"(u), "+l"(v), "+l"(w), "+l"(logz0)::"memory");
+    // wait for what is before in the stream, then let the stencil kernel, next in it, launch
+    // right away.  Velocity and log z0 may be written while this launch waits, so they take
+    // ordinary loads, which the wait orders; records and runs are as init left them
+    asm volatile("griddepcontrol.wait;" ::: "memory");
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     T acc[kStatVals];
     stats_identity(acc);
-    auto band = [&](int64_t t) {
-        return band_model<T, VEL>(mm.rec, t, t < mm.nb_w, u, v, w, mm.nx, mm.ny, (int64_t)mm.nx * mm.ny, logz0,
-                                  mm.log_phi_c, mm.kappa2);
-    };
     const int64_t nrec = mm.nb_w + mm.nb_uv;
     const int64_t stride = (int64_t)gridDim.x * blockDim.x;
     const int64_t tid = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
@@ -936,8 +930,8 @@ __global__ void __launch_bounds__(256) k_wall(KParams<T> p)
     for (int64_t t0 = tid; t0 < nrec; t0 += 2 * stride) {
         const int64_t t1 = t0 + stride;
         BandOut<T> a, b;
-        a = band(t0);
-        if (t1 < nrec) b = band(t1);
+        a = band_of<T, VEL>(mm, t0);
+        if (t1 < nrec) b = band_of<T, VEL>(mm, t1);
         store_band(mm, a, t0 < mm.nb_w);
         stats_add(acc, t0 < mm.nb_w ? 0 : 1, a.tw, a.ur);
         if (t1 < nrec) {
@@ -1793,10 +1787,15 @@ constexpr int kDirectPlain = 0, kDirectAfter = 1, kDirectSplit = 2;
 // clean chunks come first and start at once, those of dirty chunks wait for the wall
 // kernel, and the tail's blocks apply the body mask (Eq. 27) and convert the
 // statistics after the same wait.  Batch: the blocks of all members, clean ones
-// first.  NC: loads through the read-only path (hill step 207 -> 183 us: the compiler
-// keeps more of them in flight).  Not where a 32-byte sector holds values of two
-// levels: an SM's cache may then keep what a clean block read of it from before the
-// wall kernel wrote the dirty level's part.
+// first.  NC: clean blocks load through the read-only path (hill step 207 us with
+// ordinary loads throughout, 184 so: the compiler keeps more of them in flight).
+// Nothing writes what they read while the launch runs: it starts once every block of
+// the wall kernel has seen the end of what is before that one, and the wall kernel
+// writes no level that a clean block reads.
+// Dirty levels are written during the launch, so their blocks take ordinary loads,
+// which the wait orders.  Not where a 32-byte sector holds values of two levels: an
+// SM's cache may then keep what a clean block read of it from before the wall kernel
+// wrote the dirty level's part.
 template <typename T, typename VEL, int V, int KIND, bool NC, typename Batch>
 __global__ void __launch_bounds__(kDirectThreads, (kDirectBlocks<T, V>))
     k_direct(const __grid_constant__ KParams<T> p, const __grid_constant__ Batch batch)
@@ -1855,9 +1854,7 @@ __global__ void __launch_bounds__(kDirectThreads, (kDirectBlocks<T, V>))
     // what follows this launch in the stream relies on the wall kernel's end as well
     if (AFTER && (dirty || blockIdx.x == gridDim.x - 1)) wait_wall_kernel();
     if (ly >= by || i >= nx || j >= ny) return;
-    int k0 = c * kc;
-    asm volatile("" : "+r"(k0)::"memory");      // no read-only load moves ahead of the wait
-    const int k1 = min(k0 + kc, nz), plane = nx * ny;
+    const int k0 = c * kc, k1 = min(k0 + kc, nz), plane = nx * ny;
     const int im = (i == 0) ? nx - 1 : i - 1, ip = (i + V == nx) ? 0 : i + V;
     const int jm = (j == 0) ? ny - 1 : j - 1, jp = (j + 1 == ny) ? 0 : j + 1;
     const int at = j * nx + i, atm = jm * nx + i, atp = jp * nx + i, left = j * nx + im, right = j * nx + ip;
@@ -1868,54 +1865,59 @@ __global__ void __launch_bounds__(kDirectThreads, (kDirectBlocks<T, V>))
 #pragma unroll
         for (int a = 0; a < 6; ++a) q[a] = own ? p.one.tau[a] : p.one.tin[a];
     };
-    choose(k0);
-    W xz_k = ldv<NC, T, V>(q[4] + k0 * plane + at);
-    W yz_k = ldv<NC, T, V>(q[5] + k0 * plane + at);
-    W zz_km;
-    for (int e = 0; e < V; ++e) zz_km.v[e] = T(0);
-    if (k0 > 0) zz_km = ldv<NC, T, V>(q[3] + (k0 - 1) * plane + at);
-    for (int k = k0; k < k1; ++k) {
-        choose(k);
-        const bool top = k == nz - 1;
-        const int o = k * plane, up = top ? o : o + plane;
-        Level<T, V> l;
-        l.xx = ldv<NC, T, V>(q[0] + o + at);
-        l.xxl = ld1<NC>(q[0] + o + left);
-        l.xxr = ld1<NC>(q[0] + o + right);
-        l.xy = ldv<NC, T, V>(q[1] + o + at);
-        l.xyl = ld1<NC>(q[1] + o + left);
-        l.xyr = ld1<NC>(q[1] + o + right);
-        l.xyjm = ldv<NC, T, V>(q[1] + o + atm);
-        l.xyjp = ldv<NC, T, V>(q[1] + o + atp);
-        l.yyjm = ldv<NC, T, V>(q[2] + o + atm);
-        l.yyjp = ldv<NC, T, V>(q[2] + o + atp);
-        l.yzjm = ldv<NC, T, V>(q[5] + o + atm);
-        l.yzjp = ldv<NC, T, V>(q[5] + o + atp);
-        l.xzl = ld1<NC>(q[4] + o + left);
-        l.xzr = ld1<NC>(q[4] + o + right);
-        l.zz = ldv<NC, T, V>(q[3] + o + at);
-        l.xz_kp = ldv<NC, T, V>(q[4] + up + at);
-        l.yz_kp = ldv<NC, T, V>(q[5] + up + at);
-        W Fx, Fy, Fz;
-#pragma unroll
-        for (int e = 0; e < V; ++e) {
-            const T xxm = e == 0 ? l.xxl : l.xx.v[e - 1], xxp = e == V - 1 ? l.xxr : l.xx.v[e + 1];
-            const T xym = e == 0 ? l.xyl : l.xy.v[e - 1], xyp = e == V - 1 ? l.xyr : l.xy.v[e + 1];
-            const T xzm = e == 0 ? l.xzl : xz_k.v[e - 1], xzp = e == V - 1 ? l.xzr : xz_k.v[e + 1];
-            const T vx = divergence(xxp - xxm, cx, l.xyjp.v[e] - l.xyjm.v[e], cy, l.xz_kp.v[e] - xz_k.v[e], cz);
-            const T vy = divergence(xyp - xym, cx, l.yyjp.v[e] - l.yyjm.v[e], cy, l.yz_kp.v[e] - yz_k.v[e], cz);
-            const T vz = divergence(xzp - xzm, cx, l.yzjp.v[e] - l.yzjm.v[e], cy, l.zz.v[e] - zz_km.v[e], cz);
-            Fx.v[e] = top ? T(0) : vx;
-            Fy.v[e] = top ? T(0) : vy;
-            Fz.v[e] = (top || k == 0) ? T(0) : vz;
+    auto march = [&](auto read_only) {
+        constexpr bool RO = decltype(read_only)::value;
+        choose(k0);
+        W xz_k = ldv<RO, T, V>(q[4] + k0 * plane + at);
+        W yz_k = ldv<RO, T, V>(q[5] + k0 * plane + at);
+        W zz_km;
+        for (int e = 0; e < V; ++e) zz_km.v[e] = T(0);
+        if (k0 > 0) zz_km = ldv<RO, T, V>(q[3] + (k0 - 1) * plane + at);
+        for (int k = k0; k < k1; ++k) {
+            choose(k);
+            const bool top = k == nz - 1;
+            const int o = k * plane, up = top ? o : o + plane;
+            Level<T, V> l;
+            l.xx = ldv<RO, T, V>(q[0] + o + at);
+            l.xxl = ld1<RO>(q[0] + o + left);
+            l.xxr = ld1<RO>(q[0] + o + right);
+            l.xy = ldv<RO, T, V>(q[1] + o + at);
+            l.xyl = ld1<RO>(q[1] + o + left);
+            l.xyr = ld1<RO>(q[1] + o + right);
+            l.xyjm = ldv<RO, T, V>(q[1] + o + atm);
+            l.xyjp = ldv<RO, T, V>(q[1] + o + atp);
+            l.yyjm = ldv<RO, T, V>(q[2] + o + atm);
+            l.yyjp = ldv<RO, T, V>(q[2] + o + atp);
+            l.yzjm = ldv<RO, T, V>(q[5] + o + atm);
+            l.yzjp = ldv<RO, T, V>(q[5] + o + atp);
+            l.xzl = ld1<RO>(q[4] + o + left);
+            l.xzr = ld1<RO>(q[4] + o + right);
+            l.zz = ldv<RO, T, V>(q[3] + o + at);
+            l.xz_kp = ldv<RO, T, V>(q[4] + up + at);
+            l.yz_kp = ldv<RO, T, V>(q[5] + up + at);
+            W Fx, Fy, Fz;
+    #pragma unroll
+            for (int e = 0; e < V; ++e) {
+                const T xxm = e == 0 ? l.xxl : l.xx.v[e - 1], xxp = e == V - 1 ? l.xxr : l.xx.v[e + 1];
+                const T xym = e == 0 ? l.xyl : l.xy.v[e - 1], xyp = e == V - 1 ? l.xyr : l.xy.v[e + 1];
+                const T xzm = e == 0 ? l.xzl : xz_k.v[e - 1], xzp = e == V - 1 ? l.xzr : xz_k.v[e + 1];
+                const T vx = divergence(xxp - xxm, cx, l.xyjp.v[e] - l.xyjm.v[e], cy, l.xz_kp.v[e] - xz_k.v[e], cz);
+                const T vy = divergence(xyp - xym, cx, l.yyjp.v[e] - l.yyjm.v[e], cy, l.yz_kp.v[e] - yz_k.v[e], cz);
+                const T vz = divergence(xzp - xzm, cx, l.yzjp.v[e] - l.yzjm.v[e], cy, l.zz.v[e] - zz_km.v[e], cz);
+                Fx.v[e] = top ? T(0) : vx;
+                Fy.v[e] = top ? T(0) : vy;
+                Fz.v[e] = (top || k == 0) ? T(0) : vz;
+            }
+            stv(fq[0] + o + at, Fx);
+            stv(fq[1] + o + at, Fy);
+            stv(fq[2] + o + at, Fz);
+            xz_k = l.xz_kp;
+            yz_k = l.yz_kp;
+            zz_km = l.zz;
         }
-        stv(fq[0] + o + at, Fx);
-        stv(fq[1] + o + at, Fy);
-        stv(fq[2] + o + at, Fz);
-        xz_k = l.xz_kp;
-        yz_k = l.yz_kp;
-        zz_km = l.zz;
-    }
+    };
+    if (NC && !dirty) march(std::true_type{});
+    else march(std::integral_constant<bool, NC && !AFTER>{});
 }
 
 constexpr int kMaxDynSmem = 200 * 1024;
