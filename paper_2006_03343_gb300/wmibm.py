@@ -7,6 +7,7 @@ raises: there is no fallback path.
 """
 from __future__ import annotations
 
+import contextlib
 import ctypes
 import os
 from typing import Optional, Sequence
@@ -405,10 +406,10 @@ class Handle:
         for t in (*tau, *f):
             self._field(t)
         ptrs, fp = _ptrs(tau), [_dptr(t) for t in f]
-        work = torch.empty(int(self._L.wmibm_stage_work_bytes(self._h, ptrs, *fp)), dtype=torch.uint8,
-                           device=self.device)
-        if stream is not None:
-            work.record_stream(stream)
+        # allocated on the stream that uses it: a block that was freed on another one may still be in use there
+        with contextlib.nullcontext() if stream is None else torch.cuda.stream(stream):
+            work = torch.empty(int(self._L.wmibm_stage_work_bytes(self._h, ptrs, *fp)), dtype=torch.uint8,
+                               device=self.device)
         self._check(self._L.wmibm_wall_stress_force_from(self._h, _dptr(u), _dptr(v), _dptr(w), ptrs, _dptr(work),
                                                          work.numel(), *fp, None if stats is None else _dptr(stats),
                                                          _stream_ptr(stream)))
