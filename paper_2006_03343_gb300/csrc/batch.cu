@@ -152,7 +152,7 @@ int upload_members(wmibm_batch *b, const wmibm_member_fields *fields, cudaStream
         mm.run_off = run_off;
         mm.body_off = body_off;
         direct_tile(mm, 16 / (int)sizeof(T), 0, 0, kc, 0);
-        b->offsets.whole = (m == 0 || b->offsets.whole) && whole_sectors(mm);
+        mm.whole = whole_sectors(mm);
         b->offsets.clean[m] = (int32_t)clean;
         b->offsets.dirty[m] = (int32_t)dirty;
         const int64_t tiles = (int64_t)mm.gx * mm.gy;

@@ -21,6 +21,7 @@ struct Member {
     // direct-load stencil: vectors per block row, rows per block, tiles along x and y, levels per
     // chunk, and the chunks [dc0, dc0 + dcn) that hold dirty levels
     int32_t bx, by, gx, gy, kc, dc0, dcn;
+    int32_t whole;                // no 32-byte sector of the stresses holds values of two levels
     const void *rec;              // band records (w-band first)
     int64_t nb_w, nb_uv, r_off;   // band counts; first index in the record space
     int64_t nzc_w, nzc_uv;        // band nodes whose sample point's level is clamped (reported in the stats)
@@ -92,7 +93,6 @@ constexpr int kMaxBatchMembers = 256;
 // kernel parameter: the look-up runs on the constant bank).
 struct DirectBatch {
     int32_t clean[kMaxBatchMembers + 1], dirty[kMaxBatchMembers + 1];
-    int32_t whole;              // no 32-byte sector of any member's stresses holds values of two levels
 };
 
 template <typename T>

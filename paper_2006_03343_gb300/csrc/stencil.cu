@@ -1787,20 +1787,22 @@ constexpr int kDirectPlain = 0, kDirectAfter = 1, kDirectSplit = 2;
 // clean chunks come first and start at once, those of dirty chunks wait for the wall
 // kernel, and the tail's blocks apply the body mask (Eq. 27) and convert the
 // statistics after the same wait.  Batch: the blocks of all members, clean ones
-// first.  NC: clean blocks load through the read-only path (hill step 207 us with
-// ordinary loads throughout, 184 so: the compiler keeps more of them in flight).
+// first.  On rows of whole vectors clean blocks load through the read-only path (hill
+// step 207 us with ordinary loads throughout, 184 so: the compiler keeps more of them in flight).
 // Nothing writes what they read while the launch runs: it starts once every block of
 // the wall kernel has seen the end of what is before that one, and the wall kernel
 // writes no level that a clean block reads.
 // Dirty levels are written during the launch, so their blocks take ordinary loads,
-// which the wait orders.  Not where a 32-byte sector holds values of two levels: an
-// SM's cache may then keep what a clean block read of it from before the wall kernel
-// wrote the dirty level's part.
-template <typename T, typename VEL, int V, int KIND, bool NC, typename Batch>
+// which the wait orders.  Not where a 32-byte sector holds values of two levels (the
+// member's `whole` is 0): an SM's cache may then keep what a clean block read of it from
+// before the wall kernel wrote the dirty level's part.  The flag is part of the
+// descriptor, so that a captured batch step follows fields set after the capture.
+template <typename T, typename VEL, int V, int KIND, typename Batch>
 __global__ void __launch_bounds__(kDirectThreads, (kDirectBlocks<T, V>))
     k_direct(const __grid_constant__ KParams<T> p, const __grid_constant__ Batch batch)
 {
     constexpr bool BATCH = !std::is_same<Batch, NoBatch>::value, AFTER = KIND != kDirectPlain;
+    constexpr bool NC = V * sizeof(T) == 16;
     using W = Vec<T, V>;
     int b = blockIdx.x;
     const int t = threadIdx.x;
@@ -1820,7 +1822,7 @@ __global__ void __launch_bounds__(kDirectThreads, (kDirectBlocks<T, V>))
     // the member's arrays and shape: kernel parameters, or (BATCH) registers
     const T *q[6];
     T *fq[3];
-    int nx, ny, nz, bx, by, gx, gy, kc, dc0, dcn;
+    int nx, ny, nz, bx, by, gx, gy, kc, dc0, dcn, whole;
     T cx, cy, cz;
     auto take = [&](const Member<T> &m) {
 #pragma unroll
@@ -1829,6 +1831,7 @@ __global__ void __launch_bounds__(kDirectThreads, (kDirectBlocks<T, V>))
         for (int a = 0; a < 3; ++a) fq[a] = m.f[a];
         nx = m.nx; ny = m.ny; nz = m.nz;
         bx = m.bx; by = m.by; gx = m.gx; gy = m.gy; kc = m.kc; dc0 = m.dc0; dcn = m.dcn;
+        whole = m.whole;
         cx = m.cx; cy = m.cy; cz = m.cz;
     };
     if constexpr (BATCH) {
@@ -1916,8 +1919,8 @@ __global__ void __launch_bounds__(kDirectThreads, (kDirectBlocks<T, V>))
             zz_km = l.zz;
         }
     };
-    if (NC && !dirty) march(std::true_type{});
-    else march(std::integral_constant<bool, NC && !AFTER>{});
+    if (NC && (!AFTER || (!dirty && whole))) march(std::integral_constant<bool, NC>{});
+    else march(std::false_type{});
 }
 
 constexpr int kMaxDynSmem = 200 * 1024;
@@ -2138,7 +2141,7 @@ int launch_wall_single(wmibm_handle *h, void *const tau[6], const void *u, const
 
 // The direct-load stencil over p's member(s): its grid, then the launch.  body_total,
 // do_mask and emit_stats are the tail's work; pdl: the wall kernel comes just before.
-template <typename T, typename VEL, int V, int KIND, bool NC, typename Batch>
+template <typename T, typename VEL, int V, int KIND, typename Batch>
 int launch_direct(wmibm_handle *h, KParams<T> &p, const Batch &batch, bool pdl, cudaStream_t stream)
 {
     const int64_t want = (p.body_total + 2 * kDirectThreads - 1) / (2 * kDirectThreads);
@@ -2154,7 +2157,7 @@ int launch_direct(wmibm_handle *h, KParams<T> &p, const Batch &batch, bool pdl, 
     attr[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
     cfg.numAttrs = KIND != kDirectPlain && pdl ? 1 : 0;
-    return cuda_status(h, cudaLaunchKernelEx(&cfg, k_direct<T, VEL, V, KIND, NC, Batch>, p, batch), "k_direct launch");
+    return cuda_status(h, cudaLaunchKernelEx(&cfg, k_direct<T, VEL, V, KIND, Batch>, p, batch), "k_direct launch");
 }
 
 // Values per vector that every row of these arrays is aligned for.
@@ -2181,16 +2184,13 @@ int direct_single(wmibm_handle *h, KParams<T> &p, bool pdl, cudaStream_t stream)
     if (tiles * chunks > INT32_MAX / 2) return set_error(h, WMIBM_EINVAL, "grid too large for the force launch");
     p.clean_blocks = (int32_t)(tiles * (chunks - p.one.dcn));
     p.dirty_blocks = (int32_t)(tiles * p.one.dcn);
+    p.one.whole = whole_sectors(p.one);
     constexpr int kWide = 16 / (int)sizeof(T);
-    if (v == kWide) {
-        if (KIND == kDirectPlain || whole_sectors(p.one))
-            return launch_direct<T, VEL, kWide, KIND, true>(h, p, NoBatch{}, pdl, stream);
-        return launch_direct<T, VEL, kWide, KIND, false>(h, p, NoBatch{}, pdl, stream);
-    }
+    if (v == kWide) return launch_direct<T, VEL, kWide, KIND>(h, p, NoBatch{}, pdl, stream);
     if constexpr (sizeof(T) == 4) {
-        if (v == 2) return launch_direct<T, VEL, 2, KIND, false>(h, p, NoBatch{}, pdl, stream);
+        if (v == 2) return launch_direct<T, VEL, 2, KIND>(h, p, NoBatch{}, pdl, stream);
     }
-    return launch_direct<T, VEL, 1, KIND, false>(h, p, NoBatch{}, pdl, stream);
+    return launch_direct<T, VEL, 1, KIND>(h, p, NoBatch{}, pdl, stream);
 }
 
 template <typename T, typename VEL>
@@ -2588,11 +2588,8 @@ int batch_launch_direct(wmibm_handle *h0, const Member<T> *dev_members, int nmem
     int st = launch_wall_batch<T, VEL>(h0, p, c, 0, stream);
     if (st) return st;
     constexpr int V = 16 / (int)sizeof(T);
-    if (nmembers == 1)
-        return offsets.whole ? launch_direct<T, VEL, V, kDirectAfter, true>(h0, p, NoBatch{}, true, stream)
-                             : launch_direct<T, VEL, V, kDirectAfter, false>(h0, p, NoBatch{}, true, stream);
-    return offsets.whole ? launch_direct<T, VEL, V, kDirectAfter, true>(h0, p, offsets, true, stream)
-                         : launch_direct<T, VEL, V, kDirectAfter, false>(h0, p, offsets, true, stream);
+    if (nmembers == 1) return launch_direct<T, VEL, V, kDirectAfter>(h0, p, NoBatch{}, true, stream);
+    return launch_direct<T, VEL, V, kDirectAfter>(h0, p, offsets, true, stream);
 }
 
 template int batch_launch_direct<float, float>(wmibm_handle *, const Member<float> *, int, const KParams<float> &,
