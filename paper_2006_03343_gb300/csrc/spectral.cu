@@ -44,6 +44,9 @@ constexpr int kSpecBudget = 3300;       // complex elements per shared buffer ai
 // units, above it their second reads miss L2 (hill, FP32: 12 / 24 / 32 / 48 / 72 MB: 967 /
 // 742 / 761 / 789 / 797 us).
 constexpr double kSpecChunkBytes = 24.0 * 1024 * 1024;
+// limit of a block's shared memory: one value for every grid, as the limit belongs to the
+// process and other threads may be launching
+constexpr int kSpecSmemMax = 224 * 1024;
 
 struct SpecState {
     int lognx, logny;
@@ -814,8 +817,7 @@ int upload_tables(wmibm_handle *h, SpecState *s, cudaStream_t stream)
 template <typename T>
 int run_spectral(wmibm_handle *h, const SpecParams<T> &p, const SpecState *s, cudaStream_t stream)
 {
-    cudaError_t e = cudaFuncSetAttribute(k_spectral<T>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         (int)s->smem);
+    cudaError_t e = cudaFuncSetAttribute(k_spectral<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSpecSmemMax);
     if (e != cudaSuccess) return cuda_status(h, e, "k_spectral shared memory");
     int per_sm = 0;
     e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_spectral<T>, kSpecThreads, s->smem);

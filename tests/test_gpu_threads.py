@@ -78,7 +78,7 @@ def threads(tmp_path_factory):
     return ctypes.CDLL(str(d / "threads.so"))
 
 
-ENTRIES = ["sgs_stress", "sgs_force"]
+ENTRIES = ["sgs_stress", "sgs_force", "force_spectral"]
 
 
 @pytest.mark.parametrize("dtype", ["f32", "f64"])
