@@ -405,7 +405,9 @@ int wmibm_wall_stress_noalloc(wmibm_handle *h, const void *u, const void *v, con
  * wmibm_wall_stress_force and batch step of this handle computes C per node
  * from it.  The first call also builds the transpose of the band records'
  * trilinear gathers (16 entries per band node; it allocates and synchronizes
- * `stream`), so make it before any stream capture.
+ * `stream`), so make it before any stream capture.  While it builds it takes
+ * another 8 bytes per grid node of device memory, or, in more passes, as little
+ * as 4 MB where that much is not free.
  * Errors: EINVAL (misaligned logz0, more than 2^27 band nodes), ESTATE,
  * ENOMEM, ECUDA.
  */

@@ -14,6 +14,8 @@
 //      (record, corner) order; per band cell: dL/ds = w-band part + uv-band part.
 // No atomics: every output element is written by one thread in a fixed order,
 // so the result is deterministic.
+#include <algorithm>
+
 #include "band.cuh"
 
 using namespace wmibm;
@@ -236,40 +238,49 @@ __global__ void __launch_bounds__(kThreads) k_adjoint_gather(AdjParams<T> p)
 // the entries go to their node in any order and each node's few are sorted.  (Sorting
 // all entries on the host took 32 ms for the 131,072 records of 256 x 128 x 128
 // hills; this form, with its allocations, under 2 ms.)
+// The slots take 8 bytes a node while the map is built.  Where that is not to be had, the
+// chunks of slots are gone through in windows, whose entries are counted once for the
+// totals and once more for the places: a window of 4 MB is asked for at last.
 constexpr int kMapChunk = 4096;                 // slots per block of the scan
 constexpr int kMapPer = kMapChunk / kThreads;   // and per thread
+constexpr int64_t kMapWindow = 256;             // chunks of the smallest window
 
-// Slot of corner c of record r on grid g (0: uv, 1: w).
+// Slot of corner c of record r on grid g (0: uv, 1: w), each grid's from a new chunk on.
 template <typename T>
-__device__ __forceinline__ int64_t map_slot(const void *rec, int64_t r, int g, int c, int32_t nx, int32_t ny, int64_t n)
+__device__ __forceinline__ int64_t map_slot(const void *rec, int64_t r, int g, int c, int32_t nx, int32_t ny,
+                                            int64_t per_grid)
 {
     const int4 ix = __ldg(&reinterpret_cast<const typename RecOf<T>::type *>(rec)[r].ix);
     const int64_t plane = (int64_t)nx * ny;
     const int64_t di = (ix.w & 1) ? 1 - nx : 1;
     const int64_t dj = (ix.w & 2) ? (int64_t)(1 - ny) * nx : nx;
-    return g * n + (g ? ix.z : ix.y) + ((c & 1) ? di : 0) + ((c & 2) ? dj : 0) + ((c & 4) ? plane : 0);
+    return g * per_grid * kMapChunk + (g ? ix.z : ix.y) + ((c & 1) ? di : 0) + ((c & 2) ? dj : 0) +
+           ((c & 4) ? plane : 0);
 }
 
-// One thread per record, grid and corner.  FILL = false: counts the entries of each
-// slot; true: takes the slot's next place for the entry.
+// One thread per record, grid and corner; slots holds those of chunks [c0, c1).
+// FILL = false: counts the entries of each slot; true: takes the slot's next place for
+// the entry.
 template <typename T, bool FILL>
 __global__ void __launch_bounds__(kThreads) k_map_entries(const void *rec, int64_t nrec, int32_t nx, int32_t ny,
-                                                          int64_t n, int32_t *slots, int32_t *ent)
+                                                          int64_t per_grid, int64_t c0, int64_t c1, int32_t *slots,
+                                                          int32_t *ent)
 {
     const int64_t t = (int64_t)blockIdx.x * kThreads + threadIdx.x;
     if (t >= 16 * nrec) return;
     const int c = (int)(t & 7), g = (int)((t >> 3) & 1);
     const int64_t r = t >> 4;
-    const int32_t at = atomicAdd(slots + map_slot<T>(rec, r, g, c, nx, ny, n), 1);
+    const int64_t slot = map_slot<T>(rec, r, g, c, nx, ny, per_grid) - c0 * kMapChunk;
+    if (slot < 0 || slot >= (c1 - c0) * kMapChunk) return;
+    const int32_t at = atomicAdd(slots + slot, 1);
     if (FILL) ent[at] = (int32_t)(r * 8 + c);
 }
 
-// A thread's slots of chunk blockIdx.x: [first, first + count) of one grid's n slots.
-__device__ __forceinline__ void map_range(int64_t n, int64_t per_grid, int64_t &first, int &count)
+// A thread's nodes of chunk c, [first, first + count) of its grid's n.
+__device__ __forceinline__ void map_range(int64_t n, int64_t per_grid, int64_t c, int64_t &first, int &count)
 {
-    const int64_t g = blockIdx.x / per_grid, at = (blockIdx.x - g * per_grid) * kMapChunk + threadIdx.x * kMapPer;
-    first = g * n + at;
-    count = (int)min((int64_t)kMapPer, max((int64_t)0, n - at));
+    first = (c >= per_grid ? c - per_grid : c) * kMapChunk + threadIdx.x * kMapPer;
+    count = (int)min((int64_t)kMapPer, max((int64_t)0, n - first));
 }
 
 // Exclusive prefix of v over the block (x: touched slots, y: entries); total: the block's sum.
@@ -301,35 +312,36 @@ __device__ __forceinline__ int2 block_prefix(int2 v, int2 &total)
     return before;
 }
 
-// WRITE = false: the chunk's touched slots and entries into sums; true: from the
-// chunk's prefix in sums, the keys and offsets of its touched slots, whose counts
-// become the places of their first entries.
+// One block per chunk from c0 on.  WRITE = false: the chunk's touched slots and entries
+// into sums; true: from the chunk's prefix in sums, the keys and offsets of its touched
+// slots, whose counts become the places of their first entries.
 template <bool WRITE>
-__global__ void __launch_bounds__(kThreads) k_map_scan(int32_t *slots, int64_t n, int64_t per_grid, int2 *sums,
-                                                       int32_t *keys, int32_t *offs)
+__global__ void __launch_bounds__(kThreads) k_map_scan(int32_t *slots, int64_t n, int64_t per_grid, int64_t c0,
+                                                       int2 *sums, int32_t *keys, int32_t *offs)
 {
+    const int64_t c = c0 + blockIdx.x;
+    int32_t *const own = slots + (int64_t)blockIdx.x * kMapChunk + threadIdx.x * kMapPer;
     int64_t first;
     int count;
-    map_range(n, per_grid, first, count);
+    map_range(n, per_grid, c, first, count);
     int2 v = make_int2(0, 0), total;
     for (int q = 0; q < count; ++q) {
-        const int e = slots[first + q];
+        const int e = own[q];
         v.x += e != 0;
         v.y += e;
     }
     const int2 before = block_prefix(v, total);
     if (!WRITE) {
-        if (threadIdx.x == 0) sums[blockIdx.x] = total;
+        if (threadIdx.x == 0) sums[c] = total;
         return;
     }
-    int2 at = make_int2(sums[blockIdx.x].x + before.x, sums[blockIdx.x].y + before.y);
-    const int64_t base = blockIdx.x >= per_grid ? n : 0;
+    int2 at = make_int2(sums[c].x + before.x, sums[c].y + before.y);
     for (int q = 0; q < count; ++q) {
-        const int e = slots[first + q];
+        const int e = own[q];
         if (e == 0) continue;
-        keys[at.x] = (int32_t)(first + q - base);
+        keys[at.x] = (int32_t)(first + q);
         offs[at.x] = at.y;
-        slots[first + q] = at.y;
+        own[q] = at.y;
         ++at.x;
         at.y += e;
     }
@@ -389,20 +401,32 @@ __global__ void __launch_bounds__(kThreads) k_map_sort(const int32_t *offs, int6
     }
 }
 
+// The map with a window of `window` chunks' slots at a time.
 template <typename T>
-int build_map(wmibm_handle *h, cudaStream_t stream)
+cudaError_t build_map(wmibm_handle *h, int64_t window, cudaStream_t stream)
 {
     const int64_t n = h->n, entries = 16 * h->nrec, per_grid = (n + kMapChunk - 1) / kMapChunk, chunks = 2 * per_grid;
     const unsigned eblocks = (unsigned)((entries + kThreads - 1) / kThreads);
     int32_t *slots = nullptr;
     int2 *sums = nullptr;
     int2 ends[2];                               // touched slots of the uv-grid; of both, and the entries
-    cudaError_t e = dev_alloc(&slots, 2 * n * sizeof(int32_t));
+    cudaError_t e = dev_alloc(&slots, window * kMapChunk * sizeof(int32_t));
     if (e == cudaSuccess) e = dev_alloc(&sums, (chunks + 1) * sizeof(int2));
-    if (e == cudaSuccess) e = cudaMemsetAsync(slots, 0, 2 * n * sizeof(int32_t), stream);
+    auto count = [&](int64_t c0, int64_t c1) {
+        e = cudaMemsetAsync(slots, 0, (c1 - c0) * kMapChunk * sizeof(int32_t), stream);
+        if (e != cudaSuccess) return;
+        k_map_entries<T, false><<<eblocks, kThreads, 0, stream>>>(h->rec, h->nrec, h->nx, h->ny, per_grid, c0, c1, slots,
+                                                                  nullptr);
+        e = cudaGetLastError();
+    };
+    for (int64_t c0 = 0; e == cudaSuccess && c0 < chunks; c0 += window) {
+        const int64_t c1 = std::min(c0 + window, chunks);
+        count(c0, c1);
+        if (e != cudaSuccess) break;
+        k_map_scan<false><<<(unsigned)(c1 - c0), kThreads, 0, stream>>>(slots, n, per_grid, c0, sums, nullptr, nullptr);
+        e = cudaGetLastError();
+    }
     if (e == cudaSuccess) {
-        k_map_entries<T, false><<<eblocks, kThreads, 0, stream>>>(h->rec, h->nrec, h->nx, h->ny, n, slots, nullptr);
-        k_map_scan<false><<<(unsigned)chunks, kThreads, 0, stream>>>(slots, n, per_grid, sums, nullptr, nullptr);
         k_map_totals<<<1, 1024, 0, stream>>>(sums, (int)chunks);
         e = cudaGetLastError();
     }
@@ -414,10 +438,18 @@ int build_map(wmibm_handle *h, cudaStream_t stream)
     if (e == cudaSuccess) e = dev_alloc(&h->adj_offs, (m + 1) * sizeof(int32_t));
     if (e == cudaSuccess) e = dev_alloc(&h->adj_ent, entries * sizeof(int32_t));
     if (e == cudaSuccess) e = dev_alloc(&h->adj_grad, (size_t)h->nrec * 4 * sizeof(T));
+    for (int64_t c0 = 0; e == cudaSuccess && c0 < chunks; c0 += window) {
+        const int64_t c1 = std::min(c0 + window, chunks);
+        if (window < chunks) count(c0, c1);     // else the counts are still there
+        if (e != cudaSuccess) break;
+        k_map_scan<true><<<(unsigned)(c1 - c0), kThreads, 0, stream>>>(slots, n, per_grid, c0, sums, h->adj_keys,
+                                                                       h->adj_offs);
+        k_map_entries<T, true><<<eblocks, kThreads, 0, stream>>>(h->rec, h->nrec, h->nx, h->ny, per_grid, c0, c1, slots,
+                                                                 h->adj_ent);
+        e = cudaGetLastError();
+    }
     if (e == cudaSuccess) {
         const int32_t total = (int32_t)entries;
-        k_map_scan<true><<<(unsigned)chunks, kThreads, 0, stream>>>(slots, n, per_grid, sums, h->adj_keys, h->adj_offs);
-        k_map_entries<T, true><<<eblocks, kThreads, 0, stream>>>(h->rec, h->nrec, h->nx, h->ny, n, slots, h->adj_ent);
         k_map_sort<<<(unsigned)((m + kThreads - 1) / kThreads), kThreads, 0, stream>>>(h->adj_offs, m, total, h->adj_ent);
         e = cudaGetLastError();
         if (e == cudaSuccess)
@@ -433,11 +465,11 @@ int build_map(wmibm_handle *h, cudaStream_t stream)
         cudaFree(h->adj_grad);
         h->adj_keys = h->adj_offs = h->adj_ent = nullptr;
         h->adj_grad = nullptr;
-        return cuda_status(h, e, "adjoint map");
+        return e;
     }
     h->adj_m[0] = ends[0].x;
     h->adj_m[1] = m - ends[0].x;
-    return WMIBM_OK;
+    return cudaSuccess;
 }
 
 // Builds the transpose map of the trilinear gathers (once per handle).
@@ -446,7 +478,13 @@ int ensure_adjoint_map(wmibm_handle *h, cudaStream_t stream)
     if (h->adj_grad || h->nrec == 0) return WMIBM_OK;
     // entry codes (record * 8 + corner) and offsets (16 entries per record) stay below 2^31
     if (h->nrec >= (int64_t(1) << 27)) return set_error(h, WMIBM_EINVAL, "too many band records for the adjoint map");
-    return h->dtype == WMIBM_F64 ? build_map<double>(h, stream) : build_map<float>(h, stream);
+    cudaError_t e = cudaErrorMemoryAllocation;
+    for (int64_t window = 2 * ((h->n + kMapChunk - 1) / kMapChunk);; window = std::max(window / 4, kMapWindow)) {
+        e = h->dtype == WMIBM_F64 ? build_map<double>(h, window, stream) : build_map<float>(h, window, stream);
+        if (e != cudaErrorMemoryAllocation || window <= kMapWindow) break;
+        (void)cudaGetLastError();
+    }
+    return e == cudaSuccess ? WMIBM_OK : cuda_status(h, e, "adjoint map");
 }
 
 template <typename T, typename VEL>
