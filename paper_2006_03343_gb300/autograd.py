@@ -15,7 +15,8 @@ class WallStressForce(torch.autograd.Function):
     @staticmethod
     def forward(ctx, handle, u, v, w, logz0, txx, txy, tyy, tzz, txz, tyz):
         handle.set_log_z0(logz0)
-        # the stresses are read in place; views that are not contiguous go through a copy
+        # the stresses are read in place; strided and expanded views go through a dense copy (a permuted
+        # view's copy keeps its order of axes and is refused by the call, like any field that is not [nz, ny, nx])
         tau = [t if t.is_contiguous() else t.detach().clone() for t in (txx, txy, tyy, tzz, txz, tyz)]
         f = [torch.empty(handle.shape, dtype=handle.torch_dtype, device=handle.device) for _ in range(3)]
         handle.wall_stress_force_from(u, v, w, tau, f)
