@@ -1,8 +1,9 @@
 // Batched ensembles: many terrains ("members") of uneven grid sizes stepped
-// by the same two persistent launches (the wall kernel over the concatenated
-// band records, then the pipelined force + mask kernel over the concatenated
-// (member, strip, level) units).  The member descriptors live in device
-// memory, so a step is graph-capturable and replays with the same fields.
+// by the same launches: the wall kernel over the concatenated band records, then
+// the direct-load force + mask kernel over the concatenated blocks of all members,
+// or, where the batch is tuned, the pipelined kernel over the (member, strip, level)
+// units in two launches or one.  The member descriptors live in device memory, so a
+// step is graph-capturable.
 #include <stdarg.h>
 #include <stdlib.h>
 #include <string.h>
@@ -59,7 +60,7 @@ int bcuda(wmibm_batch *b, cudaError_t e, const char *what)
 
 bool aligned16(const void *p) { return ((uintptr_t)p & 15u) == 0; }
 
-// Tile shape of the batch: the widest members take `rows` x-rows per strip
+// Tile shape of the batch's pipelined forms: the widest members take `rows` x-rows per strip
 // (tuning.rows, default 4); narrower members take proportionally more rows (at
 // most 16, dividing ny) so that every member's stage carries about the same
 // bytes.  The stage slots hold the largest member's stage halves; two unless the
@@ -98,16 +99,11 @@ bool batch_config(wmibm_batch *b, StencilConfig *out, std::vector<int> *rows_out
     out->wall_warps = b->tuning.wall_warps;
     out->blocks_per_sm = b->tuning.blocks_per_sm;
     out->wall_chunk = b->tuning.wall_chunk;
-    // a batch that was never tuned also takes its units in runs of at least 16 (the
-    // autotuner's pick on the measured ensembles; a fixed share per block left a
-    // spread of about 50 us between the first and the last block)
-    const wmibm_tuning none = {};
-    const bool untuned = memcmp(&b->tuning, &none, sizeof(none)) == 0;
-    out->dyn_chunk = untuned ? 16 : b->tuning.dyn_chunk;
+    out->dyn_chunk = b->tuning.dyn_chunk;
     out->wall_grid = b->tuning.wall_grid;
     if (b->tuning.wall_grid < 0 || b->tuning.wall_grid > 32) return false;
-    // one launch (force_path 0 or 6: wall warps; 5: interleaved wall stages) or two launches (3)
     if (b->tuning.dyn_chunk < 0 || b->tuning.dyn_chunk > 4096) return false;
+    // one launch (6: wall warps; 5: interleaved wall stages) or two (0, 3)
     const int fp = b->tuning.force_path;
     if (!(fp == 0 || fp == 3 || fp == 5 || fp == 6)) return false;
     if (fp != 3 && fp != 5 && 1 + out->consumer_warps + (out->wall_warps > 0 ? out->wall_warps : 3) > 16)

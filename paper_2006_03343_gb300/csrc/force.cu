@@ -18,7 +18,7 @@ int direct_stage(wmibm_handle *h, const void *const tau[6], const void *const ow
                  void *v, void *w, const void *const gradp[3], double dt, int do_mask, bool after, bool pdl,
                  cudaStream_t stream, wmibm_band_stats *emit);
 int stencil_force(wmibm_handle *h, const void *const tau[6], void *const f[3], const StencilConfig &c,
-                  cudaStream_t stream, wmibm_band_stats *emit);
+                  cudaStream_t stream);
 
 // f = -div(tau): the direct-load kernel, or the bulk-copy pipeline where the tuning asks for it.
 int force_any(wmibm_handle *h, const void *const tau[6], void *fx, void *fy, void *fz, cudaStream_t stream)
@@ -27,7 +27,7 @@ int force_any(wmibm_handle *h, const void *const tau[6], void *fx, void *fy, voi
     StencilConfig c;
     if (use_direct(h, tau, f, &c))
         return direct_stage(h, tau, tau, f, nullptr, nullptr, nullptr, nullptr, 0.0, 0, false, false, stream, nullptr);
-    return stencil_force(h, tau, f, c, stream, nullptr);
+    return stencil_force(h, tau, f, c, stream);
 }
 
 }  // namespace wmibm

@@ -57,9 +57,6 @@ int launch(wmibm_handle *h, void *u, void *v, void *w, const void *const gradp[3
 }  // namespace
 
 namespace wmibm {
-int wall_stress_impl(wmibm_handle *h, const void *u, const void *v, const void *w, void *const tau[6],
-                     wmibm_band_stats *stats, cudaStream_t stream, const void *logz0);
-int force_any(wmibm_handle *h, const void *const tau[6], void *fx, void *fy, void *fz, cudaStream_t stream);
 bool use_direct(const wmibm_handle *h, const void *const tau[6], void *const f[3], StencilConfig *c);
 int direct_stage(wmibm_handle *h, const void *const tau[6], const void *const own[6], void *const f[3], void *u,
                  void *v, void *w, const void *const gradp[3], double dt, int do_mask, bool after, bool pdl,

@@ -865,9 +865,9 @@ int launch_spectral(wmibm_handle *h, const void *const tau[6], void *fx, void *f
 namespace wmibm {
 
 // Called once by wmibm_init: tables, counters and tile shapes of the spectral
-// forcing when nx and ny are powers of two in [2, 2048] (FP32) or [2, 1024]
-// (FP64, whose three shared buffers would not fit otherwise); otherwise the
-// handle has no spectral state and wmibm_force_spectral returns WMIBM_EINVAL.
+// forcing when nx and ny are powers of two in [2, 2048] (FP32) or [2, 1024] (FP64);
+// otherwise the handle has no spectral state and wmibm_force_spectral returns
+// WMIBM_EINVAL.
 // Errors go to the thread's last error (the handle is not returned on failure).
 int spectral_setup(wmibm_handle *h, cudaStream_t stream)
 {

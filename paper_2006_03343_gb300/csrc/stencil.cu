@@ -84,7 +84,7 @@ __device__ __forceinline__ void stg(double *p, const Pack<double> &x)
 // constant-offset loads, so that nothing is copied to local memory).
 template <typename T>
 struct ProdView {
-    const T *tau[6], *tin[6];
+    const T *tau[6];
     int32_t nx, ny, nz, ty;
 };
 
@@ -104,15 +104,11 @@ __device__ __forceinline__ void load_prod(const KParams<T> &p, int m, ProdView<T
     if (p.nmembers == 1) {
         v.tau[0] = p.one.tau[0]; v.tau[1] = p.one.tau[1]; v.tau[2] = p.one.tau[2];
         v.tau[3] = p.one.tau[3]; v.tau[4] = p.one.tau[4]; v.tau[5] = p.one.tau[5];
-        v.tin[0] = p.one.tin[0]; v.tin[1] = p.one.tin[1]; v.tin[2] = p.one.tin[2];
-        v.tin[3] = p.one.tin[3]; v.tin[4] = p.one.tin[4]; v.tin[5] = p.one.tin[5];
         v.nx = p.one.nx; v.ny = p.one.ny; v.nz = p.one.nz; v.ty = p.one.rows;
     } else {
         const Member<T> *mm = p.list + m;
         v.tau[0] = mm->tau[0]; v.tau[1] = mm->tau[1]; v.tau[2] = mm->tau[2];
         v.tau[3] = mm->tau[3]; v.tau[4] = mm->tau[4]; v.tau[5] = mm->tau[5];
-        v.tin[0] = mm->tau[0]; v.tin[1] = mm->tau[1]; v.tin[2] = mm->tau[2];
-        v.tin[3] = mm->tau[3]; v.tin[4] = mm->tau[4]; v.tin[5] = mm->tau[5];
         v.nx = mm->nx; v.ny = mm->ny; v.nz = mm->nz; v.ty = mm->rows;
     }
 }
@@ -536,10 +532,8 @@ __device__ void produce(const KParams<T> &p, T *ring_a, T *ring_b, uint64_t *ful
                 bulk_g2s(dst, base + (int64_t)jstart * nx, (uint32_t)cnt * row_bytes, &full[b]);
             }
         };
-        const bool own = it.dirty;
-        const T *const txx = own ? v.tau[0] : v.tin[0], *const txy = own ? v.tau[1] : v.tin[1];
-        const T *const tyy = own ? v.tau[2] : v.tin[2], *const tzz = own ? v.tau[3] : v.tin[3];
-        const T *const txz = own ? v.tau[4] : v.tin[4], *const tyz = own ? v.tau[5] : v.tin[5];
+        const T *const txx = v.tau[0], *const txy = v.tau[1], *const tyy = v.tau[2];
+        const T *const tzz = v.tau[3], *const txz = v.tau[4], *const tyz = v.tau[5];
         if (it.prologue) {
             const uint32_t rows = (k > 0 ? ty : 0) + ty + (ty + 2);
             mbar_arrive_expect_tx(&full[b], rows * row_bytes);
@@ -1600,10 +1594,9 @@ __global__ void __launch_bounds__(512) k_stencil(KParams<T> p)
     __syncthreads();
 
     constexpr int kFirstConsumer = 1;
-    if (MODE != kFused && p.emit_stats && blockIdx.x == 0 && threadIdx.x == 0) {
-        // statistics of the wall launch before this one (complete: stream order,
-        // or the grid dependency of a programmatic launch)
-        if (MODE == kAfterWall) wait_wall_kernel();
+    if (MODE == kAfterWall && p.emit_stats && blockIdx.x == 0 && threadIdx.x == 0) {
+        // statistics of the wall launch before this one
+        wait_wall_kernel();
         stats_emit(p.sacc, p.stats, p.one.nb_w, p.one.nb_uv, p.one.nzc_w, p.one.nzc_uv);
     }
     if (MODE == kFused && p.wall_blocks > 0 && (int)blockIdx.x < p.wall_blocks) {
@@ -2376,9 +2369,8 @@ bool stencil_config(const wmibm_handle *h, const void *const tau[6], void *const
     return true;
 }
 
-// emit: NULL, or the stats of the wall launch just before, converted by block 0.
 int stencil_force(wmibm_handle *h, const void *const tau[6], void *const f[3], const StencilConfig &c,
-                  cudaStream_t stream, wmibm_band_stats *emit)
+                  cudaStream_t stream)
 {
     if (h->dtype == WMIBM_F64) {
         KParams<double> p;
@@ -2386,8 +2378,6 @@ int stencil_force(wmibm_handle *h, const void *const tau[6], void *const f[3], c
         single_params<double>(h, p, false);
         p.stages = c.stages;
         p.ncons = c.consumer_warps;
-        p.stats = emit;
-        p.emit_stats = emit != nullptr;
         return launch_stencil<double, double, kPlain>(h, p, c, stream, false, h->nx);
     }
     KParams<float> p;
@@ -2395,8 +2385,6 @@ int stencil_force(wmibm_handle *h, const void *const tau[6], void *const f[3], c
     single_params<float>(h, p, false);
     p.stages = c.stages;
     p.ncons = c.consumer_warps;
-    p.stats = emit;
-    p.emit_stats = emit != nullptr;
     return launch_stencil<float, float, kPlain>(h, p, c, stream, false, h->nx);
 }
 
