@@ -298,7 +298,7 @@ int wmibm_wall_stress_force_from(wmibm_handle *h, const void *u, const void *v, 
                                  const void *const tau[6], void *work, int64_t work_bytes, void *fx, void *fy, void *fz,
                                  wmibm_band_stats *stats, void *stream);
 
-/* Bytes of that call's work buffer for these fields (their alignment counts) and the handle's tuning; -1 for a bad argument. */
+/* Bytes of that call's work buffer (by the handle's grid and terrain alone); -1 for a bad argument. */
 int64_t wmibm_stage_work_bytes(const wmibm_handle *h, const void *const tau[6], const void *fx, const void *fy,
                                const void *fz);
 
@@ -328,8 +328,9 @@ typedef struct wmibm_tuning {
                                  block that owns it, spread over the first half of its clean units,
                                  6 single launch with wall_warps extra warps in every block that
                                  evaluate the block's share of the band records while the producer
-                                 and consumers stream the clean units.  A batch takes 0 (two
-                                 launches, as 3), 3, 5 or 6 */
+                                 and consumers stream the clean units.  A batch takes 0 (the wall
+                                 kernel and the direct-load kernel, or with another field set as 3),
+                                 3, 5 or 6 */
     int32_t rows;             /* pipeline: rows per strip, 1, 2 or 4 */
     int32_t stages;           /* pipeline: shared-memory stages, 2..8 */
     int32_t consumer_warps;   /* pipeline: warps forming f, 1..12 */
@@ -440,8 +441,10 @@ int wmibm_backward(wmibm_handle *h, const void *const g[3], const void *const uv
  * every member, done by two launches over all members: the wall kernel over
  * the concatenated band records and solid runs, then the force + body-mask
  * kernel over the concatenated blocks of all members (or, tuned, the pipelined
- * kernel over the (member, strip, level) units).  Member descriptors (field pointers) live in device memory, so
- * a step can be captured in a CUDA graph and replayed.
+ * kernel over the (member, strip, level) units).  Member descriptors (field
+ * pointers) live in device memory, so a step can be captured in a CUDA graph and
+ * replayed; of a batch of two members or more, a replay follows fields set after
+ * the capture (a batch of one carries its fields in the launch).
  */
 typedef struct wmibm_batch wmibm_batch;
 

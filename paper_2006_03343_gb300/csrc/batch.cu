@@ -118,9 +118,9 @@ bool batch_config(wmibm_batch *b, StencilConfig *out, std::vector<int> *rows_out
 // Levels per chunk of the direct-load stencil's blocks: long chunks pay a block's
 // look-up of its member less often, short ones leave enough blocks for the launch's
 // end.  The longest of 16, 4, 2 that leaves eight waves of blocks (step in us with
-// chunks of 2 / 4 / 16 levels: 64 members of 85 M nodes 607 / 593 / 575, 5 members
-// 42.1 / 42.1 / 45.5, 6 in FP64 323 / 326 / 340; the pipelined stencil: 597, 53.6
-// and 412).
+// chunks of 2 / 4 / 16 levels: 64 members of 85 M nodes 561 / 542 / 530, 5 members
+// 49.5 / 48.3 / 49.1, 6 in FP64 369 / 374 / 388; the pipelined stencil: 592, 78.8
+// and 513).
 template <typename T>
 int direct_levels(const wmibm_batch *b)
 {

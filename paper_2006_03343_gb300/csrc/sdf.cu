@@ -393,13 +393,16 @@ __device__ __forceinline__ double level_z(const SdfParams &p, int g, int k)
     return __dmul_rn(k + (g ? 0.0 : 0.5), p.dz);
 }
 
-// Bound by the FP64 unit (58 % of its cycles on rolling terrain; the subtractions
-// z - h alone take 110 us of it at 512 x 256 x 256) and by the FP32 search beside it.
+// On rolling terrain bound by the FP64 unit (58 % of its cycles; the subtractions z - h
+// alone take 110 us of it at 512 x 256 x 256) and by the FP32 search beside it.  A single
+// hill is bound by the spread of the work: the ground around it is flat (one table for
+// all columns of a segment, and stores), and the some 290 of 4096 segments whose window
+// meets the hill do all the searching, round after round in one block each.
 // The first form gave every thread its column's near levels and evaluated whole
 // cells in FP64, so a warp paid for the union of what its lanes needed, and setting
 // up the ranges cost every thread some 60 FP64 operations.  Now the searches are
 // dense over a block, hand on single faces and edges, and those are evaluated dense
-// as well.  512 x 256 x 256, reach 4 dz: hill 908 -> 190 us, Gaussian hills 2774 ->
+// as well.  512 x 256 x 256, reach 4 dz: hill 855 -> 192 us, Gaussian hills 2774 ->
 // 567 us; 256 x 128 x 64 ridge, reach 2 dz: 499 -> 70 us (one GB300).
 //
 // A block owns one row segment of 32 columns; its 8 warps share them, warp q

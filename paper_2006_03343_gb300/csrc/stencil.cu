@@ -2112,8 +2112,8 @@ int launch_wall_single(wmibm_handle *h, void *const tau[6], const void *u, const
     // with the accumulator and emit, the wall kernel's last block converts the statistics
     p.emit_stats = (p.sacc && emit) ? 1 : 0;
     // a programmatic dependent of whatever is before it in the stream: its blocks are in
-    // place when that ends (steps back to back, 32^3 FP64 12.7 -> 10.5 us, 100 x 101 x 60
-    // 8.7 -> 6.8, cubes 256 x 128 x 128 34.1 -> 31.1, hill 512 x 256 x 256 180 -> 177).
+    // place when that ends (steps back to back, 32^3 FP64 12.7 -> 10.9 us, 100 x 101 x 60
+    // 8.6 -> 6.8, cubes 256 x 128 x 128 34.5 -> 31.7, hill 512 x 256 x 256 187 -> 184).
     // Not in a capture, whose last node need not be a kernel.
     cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
     cudaLaunchAttribute attr;

@@ -3,8 +3,8 @@
 // stencil.cu: every thread of the grid evaluates band records (trilinear
 // stencils of u, v on the uv-grid and w on the w-grid at x_c, tangential part,
 // log law, rotated stress) and warps zero the solid runs; band statistics are
-// reduced per warp and per block into an FP64 accumulator, which a one-thread
-// launch converts into the caller's stats.
+// reduced per warp and per block into an FP64 accumulator, which the last block
+// converts into the caller's stats.
 #include "internal.cuh"
 
 using namespace wmibm;

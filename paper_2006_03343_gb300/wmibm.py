@@ -567,9 +567,11 @@ class Batch:
         self._check(self._L.wmibm_batch_set_fields(self._b, arr, _stream_ptr(stream)))
 
     def set_tuning(self, **fields):
-        """Replaces the batch's tile shape and form (force_path 3: wall kernel then
-        stencil; 0 or 5: one interleaved launch); the fields given before are set
-        again, since the unit offsets depend on the rows per strip."""
+        """Replaces the batch's tile shape and form (no field set: the wall kernel, then the
+        direct-load stencil; force_path 3, or 0 with another field set: the wall kernel,
+        then the pipelined stencil; 5 and 6: one launch, with interleaved wall stages or
+        wall warps); the fields given before are set again, since the unit offsets depend
+        on the rows per strip."""
         t = Tuning()
         for k, v in fields.items():
             setattr(t, k, int(v))
